@@ -454,12 +454,15 @@ rswr_status rswr_variant_get_tiling(int32_t v, int32_t* warp_halo, int32_t* wind
  *   RSWR_VARIANT_SINGLE_ROLE      every thread loads, steps and stores windows;
  *   RSWR_VARIANT_WARP_SPECIALISED compute warps plus one producer warp that
  *                                 moves the windows (tickets, TMA, flags);
- *   RSWR_VARIANT_RESIDENT         one CTA per tile for the whole run, the
- *                                 window kept on chip and only halo strips
- *                                 exchanged between spans; a grid whose tiles
- *                                 do not all fit on the GPU at once is refused
- *                                 by rswr_run with RSWR_ENOTSUP (never a
- *                                 default variant; the autotuner tries it).
+ *   RSWR_VARIANT_RESIDENT         every warp keeps its window on chip for the
+ *                                 whole run and only halo strips are exchanged,
+ *                                 every so many spans; a grid that does not fit
+ *                                 on the GPU at once is refused by rswr_run with
+ *                                 RSWR_ENOTSUP.  A plan or batch as it was
+ *                                 created runs this way by itself when it fits
+ *                                 (same results); one whose variant, span or
+ *                                 mode was set, or chosen by the autotuner,
+ *                                 keeps to that choice.
  * RSWR_EINVAL for v out of range or kind NULL. */
 typedef enum {
     RSWR_VARIANT_SINGLE_ROLE = 0,

@@ -78,6 +78,16 @@ rswr_status validate(const rswr_problem& q)
     return RSWR_OK;
 }
 
+// A run's cut into resident warp windows.
+struct ResPlan {
+    int P = 0, S = 0, H = 0;   // points per lane, steps per exchange, halo
+    int nw = 0, per_cta = 0, grid = 0;
+    bool slack = false;        // windows leave room to put a source on a first register
+    bool linked = false;       // some problem has more than one warp
+    bool cluster = false;      // the grid is one thread-block cluster
+    double cost = 0.0;         // model: ns per step
+};
+
 struct Engine {
     int dtype = kF64;
     int form = kCanonical;
@@ -109,8 +119,16 @@ struct Engine {
     unsigned long long* d_ticket = nullptr;
     int* d_done = nullptr;
     size_t done_cap = 0;
-    void* d_xbuf = nullptr;  // resident variants: halo strips of every tile
-    size_t xbuf_cap = 0;     // bytes
+    // resident warp windows (resident.cuh): exchange slots, tables (with the
+    // host copy of what they hold) and the launch counter that tags the slots
+    void* d_xbuf = nullptr;
+    size_t xbuf_cap = 0;  // bytes
+    void* d_res = nullptr;
+    size_t res_cap = 0;  // bytes
+    std::vector<unsigned char> res_tables;
+    uint32_t res_epoch = 0;
+    std::map<std::vector<int>, ResPlan> res_plans;
+    bool chosen = false;  // variant or span set by the caller or the autotuner: runs keep to them
     DevError* d_err = nullptr;
     void* d_host_stage = nullptr;  // rswr_run_host staging
     size_t host_stage_cap = 0;
@@ -178,6 +196,7 @@ void free_engine(Engine* e)
     cudaFree(e->d_ticket);
     cudaFree(e->d_done);
     cudaFree(e->d_xbuf);
+    cudaFree(e->d_res);
     if (e->h_pstate) cudaFreeHost(e->h_pstate);
     cudaFree(e->d_err);
     cudaFree(e->d_host_stage);
@@ -277,16 +296,6 @@ rswr_status layout(Engine* e)
     }
     RSWR_CUDA(cudaMemcpy(e->d_offsets, e->h_offsets.data(), sizeof(int64_t) * e->h_offsets.size(),
                          cudaMemcpyHostToDevice));
-    if (vi.resident) {
-        const size_t xb = es * 8 * (size_t)e->H * (size_t)e->ntiles;
-        if (xb > e->xbuf_cap) {
-            cudaFree(e->d_xbuf);
-            e->d_xbuf = nullptr;
-            e->xbuf_cap = 0;
-            if (cudaMalloc(&e->d_xbuf, xb) != cudaSuccess) return fail(RSWR_ENOMEM, "halo exchange slots");
-            e->xbuf_cap = xb;
-        }
-    }
     return RSWR_OK;
 }
 
@@ -445,6 +454,7 @@ struct RunReq {
     bool mono = false;
     bool user_src = false;  // apply the engine's user point sources
     bool from_state = false;  // continue from the engine's state q[0] as it is (no level-0 set-up)
+    int64_t stop = -1;        // >= 0: take only so many of the T steps (resident runs)
     const int32_t* steps_dev = nullptr;  // the run's length on the device (<= T; SpanParams::steps_dev)
 };
 
@@ -629,7 +639,6 @@ SpanParams<Real> span_params(Engine* e, int64_t T, int nspans)
     prm.inject_span = e->inject_span;
     prm.ticket = e->d_ticket;
     prm.done = e->d_done;
-    prm.xbuf = static_cast<Real*>(e->d_xbuf);
     prm.err = e->d_err;
     prm.wait_ns = (long long)(e->wait_s * 1e9);
     return prm;
@@ -688,14 +697,7 @@ rswr_status device_work(Engine* e, const RunReq& r, int nprobe, int64_t mono_blk
         RSWR_CUDA(span_occupancy(e->variant, &bps));
         if (bps < 1) return fail(RSWR_ENOTSUP, "span kernel does not fit on an SM");
         if (nspans > 0) {
-            if (span_variant_info(e->variant).resident) {
-                // one CTA per tile for the whole run: every tile must be resident at once
-                if ((int64_t)bps * e->num_sms < e->ntiles)
-                    return fail(RSWR_ENOTSUP, "resident variant: " + std::to_string(e->ntiles) +
-                                                  " tiles do not fit on the GPU at once");
-                RSWR_CUDA(cudaMemsetAsync(e->d_done, 0, sizeof(int) * e->ntiles, s));
-                RSWR_CUDA(span_launch(e->variant, &prm, (int)e->ntiles, s));
-            } else if (e->mode == RSWR_MODE_PERSISTENT) {
+            if (e->mode == RSWR_MODE_PERSISTENT) {
                 RSWR_CUDA(cudaMemsetAsync(e->d_ticket, 0, sizeof(unsigned long long), s));
                 RSWR_CUDA(cudaMemsetAsync(e->d_done, 0, sizeof(int) * e->ntiles, s));
                 const int grid = (int)std::min<int64_t>((int64_t)bps * e->num_sms, (int64_t)nspans * e->ntiles);
@@ -813,15 +815,408 @@ rswr_status run_graph(Engine* e, const RunReq& r, int nprobe, int64_t mono_blk_o
     return RSWR_OK;
 }
 
+// ---- resident warp windows ------------------------------------------------
+
+// Points a warp owns at most: its window without the two halos.
+int res_own(int P, int H, bool slack) { return 32 * P - 2 * H - (slack ? P - 1 : 0); }
+
+// Model of the kernel's nanoseconds per step, fitted to sweeps over P, H and the
+// grid size (P 4 .. 32, H 8 .. 62, 1001 to 2^20 points): the longer of one
+// step's chain and of the work of the warps that share an SM, plus an exchange
+// every S steps (measured 0.8 us inside a cluster, 1.2 us through L2).
+double res_cost(int dtype, int P, int S, int warps_per_sm, bool linked, bool cluster)
+{
+    const double clk = 1.0 / 1.92;  // ns
+    double step;
+    if (dtype == kF64)  // 64 clocks per warp instruction on a scheduler, 16 with all four at work
+        step = clk * std::max(192.0 * P, 48.0 * P * warps_per_sm) + 12.0;
+    else
+        step = clk * std::max({60.0, 8.6 * P, ((warps_per_sm + 3) / 4) * (4.3 * P + 10.0)});
+    return step + (linked ? (cluster ? 800.0 : 1200.0) / S : 0.0);
+}
+
+// The best cut with P points per lane (P = 0: over all compiled P); false when
+// the grid does not fit on the GPU at once.  An exchange follows every m spans
+// of S steps, H = m S halo points wide (the Theorem's bound for the windows).
+bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, ResPlan* best)
+{
+    static const int Pf[] = {4, 8, 16, 32}, Pd[] = {1, 2, 4, 8, 12, 16};
+    const int* Ps = e->dtype == kF64 ? Pd : Pf;
+    const int nP = e->dtype == kF64 ? 6 : 4;
+    bool found = false;
+    for (int ip = 0; ip < nP; ++ip) {
+        const int P = Ps[ip];
+        if (want_P && P != want_P) continue;
+        for (int m = 1; m <= max_spans; ++m) {
+            const int H = m * S;
+            if (H > kResMaxHalo) break;
+            ResPlan r;
+            r.P = P;
+            r.S = H;
+            r.H = H;
+            r.slack = sources && res_own(P, H, true) >= 2 * H + 2;
+            const int own = res_own(P, H, r.slack);
+            if (own < 4) break;
+            int64_t nw = 0;
+            bool fits = true;
+            for (const ProbHost& ph : e->probs) {
+                const int64_t n = (ph.nx + own - 1) / own;
+                if (n > 1) r.linked = true;
+                if (n > 1 && ph.nx / n <= H) fits = false;  // (a piece holds more points than a halo)
+                nw += n;
+                if (nw > (int64_t)e->num_sms * 64) break;
+            }
+            const int64_t per_sm = (nw + e->num_sms - 1) / e->num_sms;
+            const int most = res_max_warps(e->dtype, P);
+            const int64_t ctas = (per_sm + most - 1) / most;  // CTAs on an SM
+            if (!fits || per_sm > 64) continue;
+            r.nw = (int)nw;
+            r.per_cta = (int)((per_sm + ctas - 1) / ctas);
+            r.grid = (r.nw + r.per_cta - 1) / r.per_cta;
+            int values = 0, occ = 0;
+            const size_t smem = res_smem_bytes(e->dtype, P, H, r.per_cta, probes ? 2 : 0, &values);
+            if (res_occupancy(e->dtype, e->form, P, 32 * r.per_cta, smem, &occ) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if ((int64_t)occ * e->num_sms < r.grid) continue;
+            r.cost = res_cost(e->dtype, P, H, (int)(ctas * r.per_cta), r.linked, false);
+            if (!found || r.cost < best->cost) {
+                *best = r;
+                found = true;
+            }
+            // the same cut as one cluster of up to 16 CTAs: exchanges through
+            // distributed shared memory, more warps on an SM
+            if (!r.linked || e->inject_tile >= 0) continue;
+            for (int per_cta = 4; per_cta <= most; per_cta += 4) {
+                const int grid = (r.nw + per_cta - 1) / per_cta;
+                if (grid > 16) continue;
+                const size_t sm = res_smem_bytes(e->dtype, P, H, per_cta, probes ? 2 : 0, &values);
+                int fit = 0;
+                if (res_occupancy(e->dtype, e->form, P, 32 * per_cta, sm, &occ) != cudaSuccess || occ < 1 ||
+                    res_clusters(e->dtype, e->form, P, grid, 32 * per_cta, sm, &fit) != cudaSuccess || fit < 1) {
+                    cudaGetLastError();
+                    continue;
+                }
+                ResPlan c = r;
+                c.cluster = true;
+                c.per_cta = per_cta;
+                c.grid = grid;
+                c.cost = res_cost(e->dtype, P, H, per_cta, true, true);
+                if (c.cost < best->cost) *best = c;
+            }
+        }
+    }
+    return found;
+}
+
+// (remembered per engine: its problems never change)
+bool res_choose(Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, ResPlan* best)
+{
+    const std::vector<int> key{want_P, S, max_spans, sources, probes, e->inject_tile >= 0};
+    auto it = e->res_plans.find(key);
+    if (it == e->res_plans.end()) {
+        ResPlan r;
+        if (!res_search(e, want_P, S, max_spans, sources, probes, &r)) r.nw = 0;
+        it = e->res_plans.emplace(key, r).first;
+    }
+    *best = it->second;
+    return best->nw > 0;
+}
+
+// Span states a resident run keeps for the adjoint sweep.
+struct ResKeep {
+    void* ck0;
+    void* ck1;
+    int64_t stride;              // elements between the states of two chunks
+    const int64_t* base;         // per problem: its first point in a state
+    bool last;
+};
+
+// One resident run: tables, one upload (skipped when the device holds the same
+// bytes already), one cooperative launch.
+template <typename Real>
+rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep* keep, cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    RSWR_CUDA(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+        return fail(RSWR_ECUDA, "runs cannot be captured: every launch carries its own exchange tag");
+    const size_t np = e->probs.size();
+    const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
+    if (r.user_src && !e->usrc.empty() && e->usrc_pitch < r.T + 1)
+        return fail(RSWR_EINVAL, "source samples hold fewer than T+1 levels");
+
+    // problems and warps
+    std::vector<ResProb<Real>> probs(np);
+    std::vector<ResWarp> warps;
+    std::vector<int32_t> first(np + 1);
+    warps.reserve(rp.nw);
+    const int own = res_own(rp.P, rp.H, rp.slack);
+    for (size_t p = 0; p < np; ++p) {
+        const ProbHost& ph = e->probs[p];
+        ResProb<Real>& d = probs[p];
+        d.off = ph.off;
+        d.base = keep ? keep->base[p] : 0;
+        d.nx = ph.nx;
+        d.fA = r.fA ? static_cast<const Real*>(r.fA) + p * (r.T + 1) : nullptr;
+        d.fB = r.fB ? static_cast<const Real*>(r.fB) + p * (r.T + 1) : nullptr;
+        d.c2 = sizeof(Real) == 8 ? (Real)ph.c2 : (Real)ph.c2f;
+        d.k = sizeof(Real) == 8 ? (Real)ph.k : (Real)ph.kf;
+        first[p] = (int32_t)warps.size();
+        const int64_t n = (ph.nx + own - 1) / own;
+        // even pieces, starting on multiples of four points (16-byte stores)
+        // where every piece still holds a strip of H points
+        const int64_t unit = n > 1 && ph.nx / n - 4 > rp.H && (ph.nx + n - 1) / n + 4 <= own ? 4 : 1;
+        for (int64_t i = 0; i < n; ++i) {
+            ResWarp w{};
+            const int64_t lo = i * ph.nx / n / unit * unit;
+            const int64_t hi = i + 1 == n ? ph.nx : (i + 1) * ph.nx / n / unit * unit;
+            w.problem = (int32_t)p;
+            w.lo = (int32_t)lo;
+            w.len = (int32_t)(hi - lo);
+            if (i > 0) w.links |= 1;
+            if (i + 1 < n) w.links |= 2;
+            w.start = w.lo - rp.H;
+            const int64_t g = (int64_t)warps.size();
+            if ((w.links & 1) && g % rp.per_cta == 0) w.links |= 4;
+            if ((w.links & 2) && g % rp.per_cta == rp.per_cta - 1) w.links |= 8;
+            warps.push_back(w);
+        }
+    }
+    first[np] = (int32_t)warps.size();
+
+    // sources, grouped by warp in the caller's order: those among a piece and
+    // the halos it needs
+    std::vector<ResSrc<Real>> srcs;
+    std::vector<std::pair<int32_t, ResSrc<Real>>> ent;
+    if (sources) {
+        auto add = [&](int64_t p, int64_t j, const Real* samples, int64_t stride) {
+            if (j <= 0 || j >= e->probs[p].nx - 1) return;  // a node's boundary data wins
+            const int64_t n = first[p + 1] - first[p], at = j * n / e->probs[p].nx;
+            for (int64_t i = std::max<int64_t>(0, at - 2); i < std::min<int64_t>(n, at + 3); ++i) {
+                const int32_t g = first[p] + (int32_t)i;
+                const ResWarp& w = warps[g];
+                if (j >= (int64_t)w.lo - rp.H && j < (int64_t)w.lo + w.len + rp.H)
+                    ent.push_back({g, ResSrc<Real>{samples, stride, (int32_t)j, 0}});
+            }
+        };
+        if (r.user_src)
+            for (const Engine::UserSrc& q : e->usrc)
+                add(q.p, q.j, static_cast<const Real*>(e->usrc_samples) + q.row * e->usrc_pitch, 1);
+        if (r.src)
+            for (size_t p = 0; p < r.js.size(); ++p)
+                if (r.js[p] >= 0) add((int64_t)p, r.js[p], static_cast<const Real*>(r.src) + p * r.src_pitch, r.src_stride);
+        std::stable_sort(ent.begin(), ent.end(), [](const std::pair<int32_t, ResSrc<Real>>& a,
+                                                    const std::pair<int32_t, ResSrc<Real>>& b) { return a.first < b.first; });
+    }
+    // where each window lies and what it holds (the kinds of resident.cuh): a
+    // grid's end window next to its node, a window with one source so that the
+    // source is a lane's first register; else nodes and sources inside
+    {
+        size_t q = 0;
+        for (size_t g = 0; g < warps.size(); ++g) {
+            ResWarp& w = warps[g];
+            w.src_begin = (int32_t)srcs.size();
+            while (q < ent.size() && ent[q].first == (int32_t)g) srcs.push_back(ent[q++].second);
+            w.src_end = (int32_t)srcs.size();
+            const int n = w.src_end - w.src_begin;
+            const bool l = w.links & 1, rt = w.links & 2;
+            w.spec = 0;
+            if (l && rt) {
+                if (n == 0) continue;
+                const int shift = (int)((((int64_t)w.start - srcs[w.src_begin].j) % rp.P + rp.P) % rp.P);
+                const bool fits = n == 1 && rp.H + shift + w.len + rp.H <= 32 * rp.P;
+                if (fits) w.start -= shift;
+                w.spec = fits ? 3 : 4;
+            } else if (l == rt || n > 0) {
+                w.spec = 4;  // (start: one halo left of the piece; its node inside)
+            } else if (!l) {
+                w.start = 1;
+                w.spec = 1;
+            } else {
+                w.start = (int32_t)(e->probs[w.problem].nx - 1 - 32 * rp.P);
+                w.spec = 2;
+            }
+        }
+    }
+
+    // probes by grid point, ranges per warp
+    std::vector<ProbeDev<Real>> probes;
+    std::vector<int32_t> prob_of;
+    {
+        std::vector<size_t> order(r.probes.size());
+        for (size_t i = 0; i < order.size(); ++i) order[i] = i;
+        std::sort(order.begin(), order.end(), [&](size_t a, size_t b) {
+            const ProbeReq &x = r.probes[a], &y = r.probes[b];
+            return x.p != y.p ? x.p < y.p : x.j < y.j;
+        });
+        size_t g = 0;
+        for (size_t i = 0; i < order.size(); ++i) {
+            const ProbeReq& q = r.probes[order[i]];
+            const ProbHost& ph = e->probs[q.p];
+            ProbeDev<Real> d{};
+            d.gidx = q.j;
+            d.out = static_cast<Real*>(q.out);
+            d.stride = q.stride;
+            d.nmax = q.nmax;
+            d.kind = q.kind;
+            if (q.scale_is_c2) d.scale = sizeof(Real) == 8 ? (Real)ph.c2 : (Real)ph.c2f;
+            else if (q.kind == 1) d.scale = sizeof(Real) == 8 ? (Real)ph.inv2dx : (Real)ph.inv2dxf;
+            else d.scale = (Real)q.scale;
+            while (g < warps.size() && (warps[g].problem < q.p ||
+                                        (warps[g].problem == q.p && (int64_t)warps[g].lo + warps[g].len <= q.j))) {
+                warps[g].probe_end = (int32_t)i;
+                if (++g < warps.size()) warps[g].probe_begin = (int32_t)i;
+            }
+            probes.push_back(d);
+        }
+        if (!order.empty()) {
+            warps[g].probe_end = (int32_t)order.size();
+            for (++g; g < warps.size(); ++g) warps[g].probe_begin = warps[g].probe_end = (int32_t)order.size();
+        }
+    }
+
+    // one table block
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t b_prob = up(sizeof(ResProb<Real>) * np), b_warp = up(sizeof(ResWarp) * warps.size());
+    const size_t b_probe = up(sizeof(ProbeDev<Real>) * probes.size()), b_src = up(sizeof(ResSrc<Real>) * srcs.size());
+    std::vector<unsigned char> tab(b_prob + b_warp + b_probe + b_src, 0);
+    std::memcpy(tab.data(), probs.data(), sizeof(ResProb<Real>) * np);
+    std::memcpy(tab.data() + b_prob, warps.data(), sizeof(ResWarp) * warps.size());
+    if (!probes.empty()) std::memcpy(tab.data() + b_prob + b_warp, probes.data(), sizeof(ProbeDev<Real>) * probes.size());
+    if (!srcs.empty())
+        std::memcpy(tab.data() + b_prob + b_warp + b_probe, srcs.data(), sizeof(ResSrc<Real>) * srcs.size());
+    if (tab.size() > e->res_cap) {
+        RSWR_CUDA(cudaStreamSynchronize(s));
+        cudaFree(e->d_res);
+        e->d_res = nullptr;
+        e->res_cap = 0;
+        e->res_tables.clear();
+        if (cudaMalloc(&e->d_res, tab.size()) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(RSWR_ENOMEM, "resident tables");
+        }
+        e->res_cap = tab.size();
+    }
+    const size_t xb = res_slot_bytes(e->dtype, rp.H) * rp.grid;
+    if (xb > e->xbuf_cap) {
+        RSWR_CUDA(cudaStreamSynchronize(s));
+        cudaFree(e->d_xbuf);
+        e->d_xbuf = nullptr;
+        e->xbuf_cap = 0;
+        if (cudaMalloc(&e->d_xbuf, xb) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(RSWR_ENOMEM, "halo exchange slots");
+        }
+        e->xbuf_cap = xb;
+        RSWR_CUDA(cudaMemsetAsync(e->d_xbuf, 0, xb, s));
+        e->res_epoch = 0;
+    }
+    if (tab != e->res_tables) {
+        RSWR_CUDA(cudaMemcpyAsync(e->d_res, tab.data(), tab.size(), cudaMemcpyHostToDevice, s));
+        e->res_tables = std::move(tab);
+    }
+    if (!r.from_state) RSWR_CUDA(cudaMemsetAsync(e->d_err, 0, sizeof(DevError), s));
+
+    ResParams<Real> prm{};
+    unsigned char* t = static_cast<unsigned char*>(e->d_res);
+    prm.problems = reinterpret_cast<const ResProb<Real>*>(t);
+    prm.warps = reinterpret_cast<const ResWarp*>(t + b_prob);
+    prm.probes = reinterpret_cast<const ProbeDev<Real>*>(t + b_prob + b_warp);
+    prm.srcs = reinterpret_cast<const ResSrc<Real>*>(t + b_prob + b_warp + b_probe);
+    prm.in0 = static_cast<const Real*>(r.q0);
+    prm.in1 = r.q0 ? static_cast<const Real*>(r.q1) : nullptr;
+    prm.out0 = static_cast<Real*>(r.out0);
+    prm.out1 = static_cast<Real*>(r.out1);
+    if (keep) {
+        prm.ck0 = static_cast<Real*>(keep->ck0);
+        prm.ck1 = static_cast<Real*>(keep->ck1);
+        prm.ck_stride = keep->stride;
+        prm.ck_last = keep->last;
+    }
+    const int64_t steps = r.stop >= 0 ? r.stop : r.T;
+    prm.T = steps;
+    prm.S = rp.S;
+    prm.H = rp.H;
+    prm.nchunks = (int32_t)((steps + rp.S - 1) / rp.S);
+    // a flux of level T at a piece's end reads a halo point, which a full chunk
+    // uses up: one more exchange before the last level is recorded
+    if (!r.probes.empty() && steps % rp.S == 0) prm.nchunks += 1;
+    prm.nwarps = (int32_t)warps.size();
+    prm.cluster = rp.cluster;
+    prm.inject_warp = e->inject_tile;
+    prm.inject_chunk = (int32_t)((int64_t)e->inject_span * e->S / rp.S);
+    prm.xbuf = static_cast<ulonglong2*>(e->d_xbuf);
+    prm.epoch = ++e->res_epoch;
+    prm.err = e->d_err;
+    prm.wait_ns = (long long)(e->wait_s * 1e9);
+    int values = 0;
+    const size_t smem = res_smem_bytes(e->dtype, rp.P, rp.H, rp.per_cta, r.probes.empty() ? 0 : 2, &values);
+    prm.warp_values = values;
+    if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
+    RSWR_CUDA(res_launch(e->dtype, e->form, rp.P, &prm, rp.grid, 32 * rp.per_cta, smem, rp.cluster, s));
+    if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+    return RSWR_OK;
+}
+
+// Whether a run takes the resident path, and its cut.  A plan whose variant is
+// a resident one always does (or the run is refused); a plan as it was created
+// does when its grid fits on the chip; a variant, span or mode chosen by the
+// caller or the autotuner is kept to.
+rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
+{
+    *take = false;
+    const VariantInfo vi = span_variant_info(e->variant);
+    const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
+    if (r.mono || r.from_state || r.steps_dev || r.T <= 0 || r.T >= ((int64_t)1 << 31) - 256) return RSWR_OK;
+    if (vi.resident) {
+        if (!res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), rp))
+            return fail(RSWR_ENOTSUP, "resident variant: the grid does not fit on the GPU at once");
+        *take = true;
+    } else if (!e->chosen && e->mode == RSWR_MODE_PERSISTENT && e->inject_tile < 0) {
+        *take = res_choose(e, 0, e->S, kResMaxHalo, sources, !r.probes.empty(), rp);
+    }
+    return RSWR_OK;
+}
+
+// A plan on a resident variant takes the default variant for a run that the
+// resident kernel does not cover, and its own tiling back afterwards.
+struct Ticketed {
+    Engine* e;
+    int variant;
+    rswr_status st = RSWR_OK;
+    Ticketed(Engine* e_, bool needed) : e(e_), variant(-1)
+    {
+        if (!needed || !span_variant_info(e->variant).resident) return;
+        variant = e->variant;
+        e->variant = default_variant(e->dtype, e->form, e->S);
+        st = layout(e);
+    }
+    ~Ticketed()
+    {
+        if (variant < 0) return;
+        cudaDeviceSynchronize();  // the run still reads the tiling that goes
+        e->variant = variant;
+        layout(e);
+    }
+};
+
 template <typename Real>
 rswr_status run_impl(Engine* e, const RunReq& r, cudaStream_t s)
 {
+    bool res = false;
+    ResPlan rp;
+    rswr_status st = res_route(e, r, &res, &rp);
+    if (st != RSWR_OK) return st;
+    if (res) return res_run<Real>(e, r, rp, nullptr, s);
+    Ticketed ticketed(e, !r.mono && r.T > 0);
+    if (ticketed.st != RSWR_OK) return ticketed.st;
     int nprobe = 0;
     int64_t mono_blk_off = -1;
-    rswr_status st = prepare_tables<Real>(e, r, &nprobe, &mono_blk_off, s);
+    st = prepare_tables<Real>(e, r, &nprobe, &mono_blk_off, s);
     if (st != RSWR_OK) return st;
-    // resident variants launch cooperatively: directly, not from a captured graph
-    if (e->use_graph && !span_variant_info(e->variant).resident) return run_graph<Real>(e, r, nprobe, mono_blk_off, s);
+    if (e->use_graph) return run_graph<Real>(e, r, nprobe, mono_blk_off, s);
     return device_work<Real>(e, r, nprobe, mono_blk_off, s);
 }
 
@@ -892,6 +1287,8 @@ rswr_status set_variant(Engine* e, int32_t v)
     if (st != RSWR_OK) {
         e->variant = old;
         layout(e);
+    } else {
+        e->chosen = true;
     }
     return st;
 }
@@ -965,18 +1362,8 @@ rswr_status adjoint_g(Engine* e, int64_t T, const int64_t* j_r, const void* wbar
 {
     const size_t es = e->esize();
     const int np = (int)e->probs.size();
-    if (e->scratch_cap < (size_t)e->packed_len) {
-        for (int b = 0; b < 2; ++b) {
-            cudaFree(e->d_scratch[b]);
-            e->d_scratch[b] = nullptr;
-            if (cudaMalloc(&e->d_scratch[b], es * e->packed_len) != cudaSuccess) return fail(RSWR_ENOMEM, "scratch");
-        }
-        e->scratch_cap = e->packed_len;
-    }
     RunReq r;
-    r.T = T + 1;
-    r.out0 = e->d_scratch[0];
-    r.out1 = e->d_scratch[1];
+    r.T = T + 1;  // (no final state is asked for)
     r.js.assign(np, -1);
     r.src = static_cast<const char*>(wbar) + es * (T + 1);
     r.src_pitch = T + 1;
@@ -1044,13 +1431,11 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
     // the persistent FP32 sweep's free warp windows ask for their own below
     int H = (SA + 3) / 4 * 4;
     // the sweeps launch span by span or with tickets: a resident plan variant
-    // gives way to the default one of its dtype and form (but runs the
-    // checkpoint sweep itself when every span state is kept; below)
+    // gives way to the default one of its dtype and form
     const VariantInfo vplan = span_variant_info(e->variant);
-    const int v_default = default_variant(e->dtype, e->form, SA);
-    int vf = vplan.resident ? v_default : e->variant;
+    const int vf = vplan.resident ? default_variant(e->dtype, e->form, SA) : e->variant;
     if (vf < 0) return fail(RSWR_ENOTSUP, "no span kernel variant for the adjoint sweep");
-    VariantInfo fi = span_variant_info(vf);
+    const VariantInfo fi = span_variant_info(vf);
     int core_f = fi.W - 2 * H;
     int64_t pad = H + 8;
     const int64_t nspans = (T + SA - 1) / SA;
@@ -1121,39 +1506,14 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
         make_layout(ai.W - 2 * H);
         C = spacing();
     }
-    // A resident plan variant runs the checkpoint sweep when every span state
-    // is kept (one launch, the tile windows on chip, each span's core written
-    // out) and the sweep's tiles all fit on the GPU at once: on small grids the
-    // ticketed sweep is paced by one tile's chain per span.
-    bool res_sweep = false;
-    if (vplan.resident && use_ws && C == 1 && variant_takes_span(vplan, SA) && vplan.W - 2 * H >= H) {
-        const int core_r = vplan.W - 2 * H;
-        int64_t ntr = 0;
-        for (int p = 0; p < np; ++p) ntr += (e->probs[p].nx + core_r - 1) / core_r;
-        int bps_r = 0;
-        RSWR_CUDA(span_occupancy(e->variant, &bps_r));
-        if ((int64_t)bps_r * e->num_sms >= ntr) {
-            vf = e->variant;
-            fi = vplan;
-            core_f = core_r;
-            make_layout(w_ws - 2 * H);
-            C = spacing();
-            res_sweep = C == 1;
-            if (!res_sweep) {
-                vf = v_default;
-                fi = span_variant_info(vf);
-                core_f = fi.W - 2 * H;
-                make_layout(w_ws - 2 * H);
-                C = spacing();
-                if (C != 1) {
-                    use_ws = false;
-                    set_halo(H_span);
-                    make_layout(ai.W - 2 * H);
-                    C = spacing();
-                }
-            }
-        }
-    }
+    // With every span state kept, the checkpoint sweep of a grid that fits on
+    // the chip is one resident launch (an exchange per span, every span's end
+    // written out): on small grids the ticketed sweep is paced by one tile's
+    // chain per span.
+    ResPlan rp;
+    const bool res_sweep = C == 1 && nspans > 0 && T < ((int64_t)1 << 31) - 256 &&
+                           (vplan.resident || (!e->chosen && e->mode == RSWR_MODE_PERSISTENT)) &&
+                           res_choose(e, 0, SA, 1, false, keep && keep->recv, &rp);
     if (keep && C != 1) return fail(RSWR_ENOMEM, "the span states of this run do not fit in device memory");
     const int64_t nck = std::max<int64_t>(1, (nspans + C - 1) / C);
     const int64_t nstates = nck + C + 4;  // checkpoints | segment | forward work pair | adjoint pair
@@ -1170,7 +1530,7 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
     const size_t need = b_states + b_partial + b_tiles + b_prob + b_probes + b_red + b_done + b_rtmp;
     // the span states of an earlier sweep with the same inputs and layout are
     // still in the workspace: the forward sweep can be skipped
-    const Engine::KeptKey key{fA, fB, T, SA, vf, va, core_f, core_a, C, use_ws, arr, need};
+    const Engine::KeptKey key{fA, fB, T, SA, res_sweep ? -1 : vf, va, core_f, core_a, C, use_ws, arr, need};
     const bool reuse = !keep && e->kept && e->kept_key == key && need <= e->adj_mem_cap;
     if (!reuse) e->kept = false;
     if (need > e->adj_mem_cap) {
@@ -1332,32 +1692,23 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
     if (!reuse) {
     RSWR_CUDA(cudaMemsetAsync(state0(CK0), 0, 2 * arr, s));
     RSWR_CUDA(set_boundary_launch(e->dtype, e->form, state0(CK0), state1(CK0), d_pu, np, s));
-    if (res_sweep && (keep ? nspans : last_ck_span) > 0) {
-        // resident tiles: one cooperative launch over every span of the sweep
-        // (a kept forward run: all of them, the final state into state nspans)
-        SpanParams<Real> cp = fp;
-        cp.span = -1;
-        cp.nspans = (int32_t)(keep ? nspans : last_ck_span);
-        cp.ck_stride = (int64_t)(2 * arr / es);
-        cp.q0[0] = state0(CK0);
-        cp.q1[0] = state1(CK0);
-        cp.q0[1] = cp.q1[1] = nullptr;
-        cp.done = d_done;
-        const size_t xb = es * 8 * (size_t)H * (size_t)ntf;
-        if (xb > e->xbuf_cap) {
-            RSWR_CUDA(cudaStreamSynchronize(s));
-            cudaFree(e->d_xbuf);
-            e->d_xbuf = nullptr;
-            e->xbuf_cap = 0;
-            if (cudaMalloc(&e->d_xbuf, xb) != cudaSuccess) {
-                cudaGetLastError();
-                return fail(RSWR_ENOMEM, "halo exchange slots");
-            }
-            e->xbuf_cap = xb;
+    if (res_sweep) {
+        RunReq r;
+        r.fA = fA;
+        r.fB = fB;
+        r.T = T;
+        const ResKeep rk{state0(CK0), state1(CK0), (int64_t)(2 * arr / es), base.data(), !keep};
+        if (keep) {
+            r.out0 = keep->out0;
+            r.out1 = keep->out1;
+            if (keep->recv) r.probes.push_back(ProbeReq{0, keep->j_rec, 0, 1.0, keep->recv, 1, T});
+        } else {
+            r.stop = last_ck_span * SA;
         }
-        cp.xbuf = static_cast<Real*>(e->d_xbuf);
-        RSWR_CUDA(cudaMemsetAsync(d_done, 0, sizeof(int) * ntf, s));
-        RSWR_CUDA(span_launch(vf, &cp, (int)ntf, s));
+        if (keep || last_ck_span > 0) {
+            rswr_status st = res_run<Real>(e, r, rp, &rk, s);
+            if (st != RSWR_OK) return st;
+        }
     } else if (C == 1 && last_ck_span > 0) {
         // every span state is kept: the whole sweep is one persistent launch in
         // which span k reads state k and writes state k + 1 (neighbour flags as in
@@ -1391,17 +1742,13 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
         e->kept_key = key;
     }
 
+    if (keep && res_sweep) return RSWR_OK;  // (receiver and final state written by the resident run)
     if (keep) {
         // a kept forward run: the last span into the work pair, the receiver's
         // last level, the final state pair
         Real* f0 = state0(CK0);
         Real* f1 = state1(CK0);
-        if (res_sweep && nspans > 0) {
-            // the resident sweep ran every span: the final state is state nspans
-            // (the segment slot, unused when every span state is kept)
-            f0 = state0(CK0 + nspans);
-            f1 = state1(CK0 + nspans);
-        } else if (nspans > 0) {
+        if (nspans > 0) {
             const int64_t k = nspans - 1;  // C == 1: state k is checkpoint k
             rswr_status st = forward_span(k, state0(CK0 + k), state1(CK0 + k), state0(WK0), state1(WK0));
             if (st != RSWR_OK) return st;
@@ -1564,6 +1911,7 @@ rswr_status apply_choice(Engine* e, const TuneChoice& c)
         return st;
     }
     e->mode = c.mode;
+    e->chosen = true;
     return RSWR_OK;
 }
 
@@ -1618,7 +1966,7 @@ rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cu
         const VariantInfo vi = span_variant_info(v);
         if (vi.dtype != e->dtype || vi.form != e->form) continue;
         for (int S : spans) {
-            for (int mode = 0; mode < (vi.resident ? 1 : 2); ++mode) {
+            for (int mode = 0; mode < (vi.resident ? 1 : 2); ++mode) {  // (one mode for resident windows)
                 if (apply_choice(e, TuneChoice{v, mode, S}) != RSWR_OK) continue;
                 if (run_engine(e, r, s) != RSWR_OK) continue;  // warm-up (and graph capture)
                 RSWR_CUDA(cudaEventRecord(a, s));
@@ -1669,6 +2017,8 @@ template <typename Real>
 rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, const Real* q0, const Real* q1, Real* out0,
                       Real* out1, int64_t* spans, int64_t spans_cap, int64_t* nspans, double beta, cudaStream_t s)
 {
+    Ticketed ticketed(e, true);  // the spans continue from the state arrays
+    if (ticketed.st != RSWR_OK) return ticketed.st;
     const ProbHost& ph = e->probs[0];
     const int64_t nx = ph.nx, N = ph.n_sub, ov = ph.ov, el = (ov + 1) / 2, er = ov / 2;
     const size_t es = sizeof(Real);
@@ -1974,6 +2324,8 @@ rswr_status rswr_plan_set_span(rswr_plan_t plan, int32_t S)
         e->S = old;
         e->variant = oldv;
         layout(e);
+    } else {
+        e->chosen = true;
     }
     return st;
 }

@@ -87,7 +87,6 @@ struct SpanParams {
     int64_t ck_stride;           // 0: span k reads q[k & 1] and writes q[(k + 1) & 1];
                                  // > 0: span k reads q[0] + k * ck_stride and writes
                                  // q[0] + (k + 1) * ck_stride (every span state kept)
-    Real* xbuf;                  // resident variants: halo strips, [tile][span parity][side][component][H]
     const int32_t* steps_dev;    // non-null: the run's length is *steps_dev (<= T), read on the device
                                  // (the paper-literal path chooses its span there); later spans of the
                                  // launch then take no steps and pass their tiles through
@@ -187,6 +186,66 @@ struct PaperParams {
     const PaperState* st;  // non-null: n0, steps and the span come from here (n0 / steps above unused)
 };
 
+// ---- resident warp windows (resident.cuh) -------------------------------------
+
+constexpr int kResMaxHalo = 64;     // steps between two exchanges at most
+
+// One warp's piece of a problem: grid points [lo, lo + len), window from
+// `start` on.  links: 1 / 2 a left / right neighbour, 4 / 8 the same in another
+// CTA.  Probes of the owned points, sources of the window.
+struct ResWarp {
+    int32_t problem, start, lo, len;
+    int32_t probe_begin, probe_end, src_begin, src_end;
+    int32_t links, spec;  // spec: what the window holds (resident.cuh)
+    int32_t pad_[2];
+};
+
+template <typename Real>
+struct ResProb {
+    int64_t off;   // the problem's first point in the packed state arrays
+    int64_t base;  // ... in the kept span states (adjoint sweep)
+    int64_t nx;
+    const Real* fA;
+    const Real* fB;
+    Real c2, k;
+};
+
+template <typename Real>
+struct ResSrc {
+    const Real* samples;  // level n at samples[n * stride]
+    int64_t stride;
+    int32_t j, pad_;
+};
+
+template <typename Real>
+struct ResParams {
+    const ResProb<Real>* problems;
+    const ResWarp* warps;
+    const ProbeDev<Real>* probes;  // gidx: the grid point
+    const ResSrc<Real>* srcs;      // grouped by warp
+    const Real* in0;               // packed initial state (null: zero data / at rest)
+    const Real* in1;
+    Real* out0;                    // packed final state
+    Real* out1;
+    Real* ck0;                     // kept span states: chunk k ends in ck + (k + 1) * ck_stride (null: none)
+    Real* ck1;
+    int64_t ck_stride;
+    int64_t T;
+    int32_t ck_last;      // 1: the last chunk's end is kept too
+    int32_t S;            // steps of a chunk
+    int32_t H;            // halo of a window (>= S)
+    int32_t nchunks;
+    int32_t nwarps;
+    int32_t warp_values;  // shared-memory values of one warp
+    int32_t pad_;
+    int32_t inject_warp, inject_chunk;  // test hook (-1: off)
+    int32_t cluster;      // 1: the grid is one thread-block cluster
+    ulonglong2* xbuf;     // exchange slots [CTA][side][parity][H * words]
+    unsigned long long epoch;  // of this launch, part of the slots' tags
+    DevError* err;
+    long long wait_ns;
+};
+
 struct VariantInfo {
     int dtype;
     int form;
@@ -196,7 +255,7 @@ struct VariantInfo {
     int W;   // points per CTA window
     int threads;   // threads per CTA at launch (NT, or NT + a producer warp)
     int max_span;  // longest span the variant runs (0: any that fits the window)
-    int resident;  // 1: one CTA per tile for the whole run (cooperative launch, grid = tiles)
+    int resident;  // 1: every warp keeps its window for the whole run (cooperative launch, resident.cuh)
 };
 
 // span_kernel.cu
@@ -206,6 +265,16 @@ size_t span_smem_bytes(int v);
 cudaError_t span_prepare(int v);  // sets the dynamic shared-memory attribute
 cudaError_t span_occupancy(int v, int* blocks_per_sm);
 cudaError_t span_launch(int v, const void* params, int grid, cudaStream_t s);
+
+// resident_kernel.cu: P points per lane; -1 / error when (dtype, form, P) is not compiled
+size_t res_smem_bytes(int dtype, int P, int H, int warps_per_cta, int probe_rows, int* warp_values);
+int res_max_warps(int dtype, int P);      // warps of a CTA at most
+size_t res_slot_bytes(int dtype, int H);  // exchange slots of one CTA
+cudaError_t res_occupancy(int dtype, int form, int P, int threads, size_t smem, int* ctas_per_sm);
+// clusters of `grid` CTAs that fit on the GPU at once
+cudaError_t res_clusters(int dtype, int form, int P, int grid, int threads, size_t smem, int* clusters);
+cudaError_t res_launch(int dtype, int form, int P, const void* params, int grid, int threads, size_t smem,
+                       bool cluster, cudaStream_t s);
 
 // adjoint_kernel.cu
 int adj_variant_count();

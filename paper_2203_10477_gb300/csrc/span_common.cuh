@@ -551,30 +551,15 @@ struct NoRecord {
     __device__ __forceinline__ void operator()(const U&, Real, Real, int) const {}
 };
 
-// Special points in the edges-first loop (Dirichlet nodes, a point source, the
-// outside points next to the nodes; see patch_special): pre(u, s) runs before
-// step s (samples, level-n values), edges(u, n0, v0, nl, vl) patches the new
-// values of the thread's first and last register before they are shuffled,
-// interior(u, w) the registers in between after their update.
-struct NoPatch {
-    template <typename U>
-    __device__ __forceinline__ void pre(const U&, int) {}
-    template <typename U, typename Real>
-    __device__ __forceinline__ void edges(const U&, Real&, Real&, Real&, Real&) {}
-    template <typename U>
-    __device__ __forceinline__ void interior(U&, U&) {}
-};
-
-template <typename Real, int FORM, int P, typename Rec = NoRecord, typename Patch = NoPatch>
+template <typename Real, int FORM, int P, typename Rec = NoRecord>
 __device__ __forceinline__ void warp_steps_edges_first(Real (&u)[P], Real (&w)[P], Real c2, Real k, int steps,
-                                                       int lane, Rec rec = Rec{}, Patch patch = Patch{})
+                                                       int lane, Rec rec = Rec{})
 {
     static_assert(P >= 3, "edges-first order needs interior points");
     Real lft, rgt;
     warp_neighbours<Real, P>(u, lft, rgt, lane);
     for (int s = 0; s < steps; ++s) {
         rec(u, lft, rgt, s);
-        patch.pre(u, s);
         Real n0, nl, v0, vl;  // new first / last point and their second components
         Real d0 = Real(0);
         if constexpr (FORM == kIncrement) {
@@ -590,7 +575,6 @@ __device__ __forceinline__ void warp_steps_edges_first(Real (&u)[P], Real (&w)[P
             nl = rfma(c2, radd(u[P - 2], rgt), rfma(k, u[P - 1], -w[P - 1]));
             vl = u[P - 1];
         }
-        patch.edges(u, n0, v0, nl, vl);
         Real nlft = __shfl_up_sync(kFull, nl, 1);
         Real nrgt = __shfl_down_sync(kFull, n0, 1);
         if constexpr (FORM == kIncrement) {
@@ -618,126 +602,12 @@ __device__ __forceinline__ void warp_steps_edges_first(Real (&u)[P], Real (&w)[P
         w[0] = v0;
         u[P - 1] = nl;
         w[P - 1] = vl;
-        patch.interior(u, w);
         if (lane == 0) nlft = u[1];
         if (lane == 31) nrgt = u[P - 2];
         lft = nlft;
         rgt = nrgt;
     }
 }
-
-// The patch of the special points for warp_steps_edges_first, with the same
-// effect as leap_step + patch_special: a register takes, in this order, the
-// source (canonical u' += s; increment v' += s, u' = u_old + v'), the left node
-// (u' = f_A(n+1); increment v' = f_A(n+1) - f_A(n)), the outside point next to
-// it (0, 0), the right node, the outside point next to it.  Samples come from
-// the warp's chunks (f_A / f_B at level n0 + d, the source at level n0 + d + 1).
-// Whether a special point of the thread sits between its first and last
-// register (the register trees of EdgePatch::interior are needed).
-template <int P>
-__device__ __forceinline__ bool interior_special(const Special& sp)
-{
-    auto in = [](int r) { return r > 0 && r < P - 1; };
-    return in(sp.rs) || in(sp.r0) || in(sp.rm) || in(sp.r1) || in(sp.rp);
-}
-
-// INTERIOR = false: every special point of the warp sits on a thread's first
-// or last register, so interior() has nothing to do and is compiled out (the
-// register trees, which the compiler turns into predicated code that every lane
-// executes each step, are what make the patched loop slow).
-template <typename Real, int FORM, int P, typename Reload, bool INTERIOR = true>
-struct EdgePatch {
-    Special sp;
-    WarpChunk<Real>* ca;
-    WarpChunk<Real>* cb;
-    WarpChunk<Real>* cs;
-    bool wa, wb, wsrc;
-    int* cbase;       // first step of the current chunk
-    Reload* reload;   // reload(first): loads the chunk after the one starting at `first`
-    Real fa_old, fa_new, fb_old, fb_new, sval, uold_s;
-    int d;
-
-    template <typename U>
-    __device__ __forceinline__ void pre(const U& u, int s)
-    {
-        step_samples(s);
-        capture(u);
-    }
-    __device__ __forceinline__ void step_samples(int s)
-    {
-        d = s - *cbase;
-        if (d == 32) {
-            *cbase += 32;
-            ca->c0 = ca->c1;
-            cb->c0 = cb->c1;
-            cs->c0 = cs->c1;
-            (*reload)(*cbase, false);
-            d = 0;
-        }
-        fa_old = fa_new = fb_old = fb_new = sval = Real(0);
-        if (wsrc) sval = cs->get(d);
-        if (wa) {
-            fa_old = ca->get(d);
-            fa_new = ca->get(d + 1);
-        }
-        if (wb) {
-            fb_old = cb->get(d);
-            fb_new = cb->get(d + 1);
-        }
-    }
-    __device__ __forceinline__ void at(int i, Real& x, Real& y)
-    {
-        if (sp.rs == i) {
-            if constexpr (FORM == kIncrement) {
-                y = radd(y, sval);
-                x = radd(uold_s, y);
-            } else {
-                x = radd(x, sval);
-            }
-        }
-        if (sp.r0 == i) {
-            x = fa_new;
-            if constexpr (FORM == kIncrement) y = rsub(fa_new, fa_old);
-        }
-        if (sp.rm == i) x = y = Real(0);
-        if (sp.r1 == i) {
-            x = fb_new;
-            if constexpr (FORM == kIncrement) y = rsub(fb_new, fb_old);
-        }
-        if (sp.rp == i) x = y = Real(0);
-    }
-    template <typename U>
-    __device__ __forceinline__ void capture(const U& u)
-    {
-        // the level-n value of the source point (increment form)
-        if constexpr (FORM == kIncrement)
-            if (sp.rs >= 0) uold_s = reg_get<Real, P>(u, sp.rs);
-    }
-    template <typename U>
-    __device__ __forceinline__ void edges(const U& u, Real& n0, Real& v0, Real& nl, Real& vl)
-    {
-        at(0, n0, v0);
-        at(P - 1, nl, vl);
-    }
-    template <typename U>
-    __device__ __forceinline__ void interior(U& u, U& w)
-    {
-        if constexpr (!INTERIOR) return;
-        // one jump-table branch per special point held between the end registers
-        auto one = [&](int r) {
-            if (r > 0 && r < P - 1)
-                reg_switch<P>(r, [&](auto I) {
-                    constexpr int i = decltype(I)::value;
-                    at(i, u[i], w[i]);
-                });
-        };
-        one(sp.rs);
-        if (sp.r0 != sp.rs) one(sp.r0);
-        one(sp.rm);
-        if (sp.r1 != sp.rs) one(sp.r1);
-        one(sp.rp);
-    }
-};
 
 // Write the registers a thread owns, [own_lo, own_hi), back to the shared window.
 template <typename Real, int P, int KH>

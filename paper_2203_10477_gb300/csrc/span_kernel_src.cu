@@ -23,7 +23,7 @@ const void* src_kernel_WS()
 template <typename Real, int FORM, int P, int NT, int KH, int MINB>
 const void* src_kernel_RES()
 {
-    return reinterpret_cast<const void*>(&span_kernel_res<Real, FORM, P, NT, KH, MINB, true>);
+    return nullptr;  // one kernel with and without sources (resident.cuh)
 }
 
 #define RSWR_SRC_KERNEL(kind, Real, FORM, P, NT, KH, MINB) src_kernel_##kind<Real, FORM, P, NT, KH, MINB>(),
