@@ -25,8 +25,10 @@
 //   * a window is placed so that a Dirichlet node is the neighbour of its
 //     outermost point (one select a step) and a point source sits on a lane's
 //     first register (two); other cases take compares per register;
-//   * a probe's lane drops its registers into a shared row per step, and the
-//     warp turns 16 rows into one coalesced store.
+//   * a probe's window is placed so that its point is a lane's first or last
+//     register; the lane drops the value into a shared buffer every step, and the
+//     warp turns 32 levels into one coalesced store (elsewhere: rows of all the
+//     lane's registers).
 // The final state goes straight to the caller's arrays, the initial state
 // comes straight from them.
 
@@ -40,7 +42,8 @@ namespace resident {
 
 using span::kFull;
 
-constexpr int kRing = 16;  // levels of a probe row buffer
+constexpr int kRing = 16;      // levels of a probe row buffer
+constexpr int kFastRing = 32;  // levels of a buffer of probes on end registers
 
 // ---- 16-byte single-copy-atomic accesses at gpu scope ------------------------
 __device__ __forceinline__ void st_pair(ulonglong2* p, unsigned long long lo, unsigned long long hi)
@@ -62,6 +65,34 @@ __device__ __forceinline__ void ld_pair(const ulonglong2* p, unsigned long long&
 template <typename Real>
 constexpr int slot_words = sizeof(Real) == 4 ? 1 : 2;
 
+// Stores of one lane without a branch (a branch that one lane takes costs a
+// reconvergence, some 100 clocks a step on a lone warp).
+__device__ __forceinline__ void st_shared_if(bool on, const float* d, float a, float b)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.v2.f32 [%1], {%2, %3};\n\t}" ::"r"((uint32_t)on),
+                 "r"(smem_addr(d)), "f"(a), "f"(b)
+                 : "memory");
+}
+__device__ __forceinline__ void st_shared_if(bool on, const double* d, double a, double b)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.v2.f64 [%1], {%2, %3};\n\t}" ::"r"((uint32_t)on),
+                 "r"(smem_addr(d)), "d"(a), "d"(b)
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_shared_if16(bool on, const float* d, const float* x)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t"
+                 "@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t"
+                 "@p st.shared.v4.f32 [%1 + 16], {%6, %7, %8, %9};\n\t"
+                 "@p st.shared.v4.f32 [%1 + 32], {%10, %11, %12, %13};\n\t"
+                 "@p st.shared.v4.f32 [%1 + 48], {%14, %15, %16, %17};\n\t}" ::"r"((uint32_t)on),
+                 "r"(smem_addr(d)), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]),
+                 "f"(x[7]), "f"(x[8]), "f"(x[9]), "f"(x[10]), "f"(x[11]), "f"(x[12]), "f"(x[13]), "f"(x[14]),
+                 "f"(x[15])
+                 : "memory");
+}
+
 // Warps of a CTA at most: 16 (one CTA then holds an SM's whole register file),
 // 8 where a lane's points fill more than 64 registers.
 template <typename Real>
@@ -77,7 +108,8 @@ template <typename Real>
 __host__ __device__ inline size_t warp_values(int H, int P, int probe_rows)
 {
     size_t n = (size_t)128 * P + 8 * H;
-    n += (size_t)probe_rows * kRing * kRowLanes<Real>(P) * P;
+    const int row = kRing * kRowLanes<Real>(P) * P;
+    n += (size_t)probe_rows * (row > 2 * kFastRing ? row : 2 * kFastRing);
     return (n + 3) / 4 * 4;
 }
 
@@ -132,7 +164,8 @@ enum : int {
 
 // `steps` leapfrog steps of the window from level lv on.  mine: this lane's
 // shuffle (node) or register (source) takes the stream's samples.
-// rec(u, s) sees level lv + s before it is advanced; patch(u, w, u_old, s)
+// rec(u, lft, rgt, s) sees level lv + s before it is advanced (it must not shuffle
+// inside a divergent branch); patch(u, w, u_old, s)
 // patches the special points after the step (kAny).
 template <typename Real, int FORM, int P, int SPEC, typename Rec, typename Patch>
 __device__ __forceinline__ void run_steps(Real (&u)[P], Real (&w)[P], Real c2, Real k, int lv, int steps, bool mine,
@@ -156,10 +189,11 @@ __device__ __forceinline__ void run_steps(Real (&u)[P], Real (&w)[P], Real c2, R
         }
 #pragma unroll kUnroll
         for (int s = s0; s < s1; ++s) {
-            rec(u, s);
+            const Real l_old = lft, r_old = rgt;
             Real nxt = Real(0);
             if constexpr (kStream) nxt = st.after(lv + s);  // (in time for the end of this step)
             if constexpr (SPEC == kAny) {
+                rec(u, l_old, r_old, s);
                 Real uo[P];  // level n
 #pragma unroll
                 for (int i = 0; i < P; ++i) uo[i] = u[i];
@@ -192,6 +226,7 @@ __device__ __forceinline__ void run_steps(Real (&u)[P], Real (&w)[P], Real c2, R
                 add_source();
                 lft = __shfl_up_sync(kFull, n0, 1);
                 rgt = __shfl_down_sync(kFull, n0, 1);
+                rec(u, l_old, r_old, s);
                 u[0] = n0;
                 w[0] = v0;
             } else if constexpr (FORM == kIncrement) {
@@ -206,6 +241,7 @@ __device__ __forceinline__ void run_steps(Real (&u)[P], Real (&w)[P], Real c2, R
                 const Real nl = radd(u[P - 1], vl);
                 lft = __shfl_up_sync(kFull, nl, 1);
                 rgt = __shfl_down_sync(kFull, n0, 1);
+                rec(u, l_old, r_old, s);
                 Real dprev = d0;
 #pragma unroll
                 for (int i = 1; i < P - 1; ++i) {
@@ -226,6 +262,7 @@ __device__ __forceinline__ void run_steps(Real (&u)[P], Real (&w)[P], Real c2, R
                 const Real nl = rfma(c2, radd(u[P - 2], rgt), rfma(k, u[P - 1], -w[P - 1]));
                 lft = __shfl_up_sync(kFull, nl, 1);
                 rgt = __shfl_down_sync(kFull, n0, 1);
+                rec(u, l_old, r_old, s);
                 Real ul = u[0];
 #pragma unroll
                 for (int i = 1; i < P - 1; ++i) {
@@ -285,20 +322,115 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t a, int rank)
     return r;
 }
 
-// Owned points to a global array (dst: grid point 0 of the problem).
+// A window (one component) in shared memory as 16-byte units, the low bits of a
+// unit's place mixed with the next ones: neither a lane's own P points nor
+// consecutive points of the window meet bank conflicts.
+template <typename Real>
+__device__ __forceinline__ int unit_place(int unit)
+{
+    return (unit ^ ((unit >> 3) & 7)) * (int)(16 / sizeof(Real));
+}
+
+// unit_place(u0 + i), u0 = lane * (P / N): with up to 8 units per lane the mixing
+// term is the same for all of them (one exclusive-or per unit)
 template <typename Real, int P>
-__device__ __forceinline__ void store_owned(Real* dst, const Real (&v)[P], int j0, int lo, int hi)
+__device__ __forceinline__ int lane_unit(uint32_t u0, int i)
+{
+    constexpr int N = 16 / sizeof(Real);
+    if constexpr (P / N <= 8 && (P / N & (P / N - 1)) == 0)
+        return (int)(((u0 & ~7u) + (((u0 & 7u) + i) ^ ((u0 >> 3) & 7u))) * N);
+    else
+        return unit_place<Real>((int)u0 + i);
+}
+
+template <typename Real, int P>
+__device__ __forceinline__ void put_units(Real* sm, const Real (&v)[P], int lane)
 {
     constexpr int N = 16 / sizeof(Real);
     if constexpr (P % N == 0) {
-        if (j0 >= lo && j0 + P <= hi && (reinterpret_cast<uintptr_t>(dst + j0) & 15) == 0) {
-            span::regs_to_smem<Real, P>(dst + j0, v);  // (16-byte stores)
-            return;
+        using V = typename span::Vec<Real, P>::T;
+        const uint32_t u0 = (uint32_t)(lane * (P / N));
+#pragma unroll
+        for (int i = 0; i < P / N; ++i) {
+            V x;
+            x.x = v[N * i];
+            x.y = v[N * i + 1];
+            if constexpr (N == 4) {
+                x.z = v[N * i + 2];
+                x.w = v[N * i + 3];
+            }
+            *reinterpret_cast<V*>(sm + lane_unit<Real, P>(u0, i)) = x;
+        }
+    } else {  // (FP64, one point per lane)
+        sm[unit_place<Real>(lane / N) + lane % N] = v[0];
+    }
+}
+
+template <typename Real, int P>
+__device__ __forceinline__ void get_units(const Real* sm, Real (&v)[P], int lane)
+{
+    constexpr int N = 16 / sizeof(Real);
+    static_assert(P % N == 0, "whole units");
+    using V = typename span::Vec<Real, P>::T;
+    const uint32_t u0 = (uint32_t)(lane * (P / N));
+#pragma unroll
+    for (int i = 0; i < P / N; ++i) {
+        const V x = *reinterpret_cast<const V*>(sm + lane_unit<Real, P>(u0, i));
+        v[N * i] = x.x;
+        v[N * i + 1] = x.y;
+        if constexpr (N == 4) {
+            v[N * i + 2] = x.z;
+            v[N * i + 3] = x.w;
         }
     }
+}
+
+// The window's points [a, a + n) to a global array (dst: window position 0)
+// through shared memory, so that a warp's stores cover whole lines (straight
+// from the registers a store touches a 16-byte piece of 32 lines: 1.4 TB/s
+// measured).  In shared memory the window is moved up by the 0 .. N - 1 points
+// that put its units on the array's 16-byte boundaries.
+template <typename Real, int P>
+__device__ __forceinline__ void store_owned(Real* dst, const Real (&v)[P], Real* sm, int lane, int a, int n)
+{
+    constexpr int N = 16 / sizeof(Real);
+    const int off = (int)((reinterpret_cast<uintptr_t>(dst) / sizeof(Real)) & (N - 1));
+    if (off == 0 && P % N == 0) {
+        put_units<Real, P>(sm, v, lane);
+    } else {
 #pragma unroll
-    for (int i = 0; i < P; ++i)
-        if (j0 + i >= lo && j0 + i < hi) dst[j0 + i] = v[i];
+        for (int i = 0; i < P; ++i) {
+            const int p = lane * P + i + off;
+            sm[unit_place<Real>(p / N) + p % N] = v[i];
+        }
+    }
+    __syncwarp();
+    dst -= off;
+    const int b = a + off, e = b + n;                    // positions in shared memory
+    const int u0 = (b + N - 1) / N, u1 = e / N;          // whole units [u0, u1)
+    if (u0 < u1) {
+        using V = typename span::Vec<Real, P>::T;
+        // 32 units on, the mixing term changes in its third bit: two places in turn
+        const int u = u0 + lane;
+        const Real* s0 = sm + unit_place<Real>(u);
+        const Real* s1 = sm + unit_place<Real>(u + 32);
+        Real* d = dst + u * N;
+        constexpr int K = (P + N - 1) / N;
+#pragma unroll
+        for (int k = 0; k < K; k += 2) {
+            if (u + 32 * k < u1) *reinterpret_cast<V*>(d + 32 * N * k) = *reinterpret_cast<const V*>(s0 + 32 * N * k);
+            if (k + 1 < K && u + 32 * k + 32 < u1)
+                *reinterpret_cast<V*>(d + 32 * N * (k + 1)) = *reinterpret_cast<const V*>(s1 + 32 * N * k);
+        }
+    }
+    // the points before the first and after the last whole unit
+    if (u0 > u1 || u0 * N != b || u1 * N != e) {
+        const int h = u0 <= u1 ? u0 * N : e;
+        if (b + lane < h) dst[b + lane] = sm[unit_place<Real>((b + lane) / N) + (b + lane) % N];
+        const int t = u0 <= u1 ? u1 * N : e;
+        if (t + lane < e) dst[t + lane] = sm[unit_place<Real>((t + lane) / N) + (t + lane) % N];
+    }
+    __syncwarp();
 }
 
 template <typename Real, int P>
@@ -315,6 +447,253 @@ __device__ __forceinline__ void load_window(const Real* src, Real (&v)[P], int j
     for (int i = 0; i < P; ++i) v[i] = (j0 + i >= 0 && j0 + i < nx) ? src[j0 + i] : Real(0);
 }
 
+// The exchange between a warp and its two neighbours: the H owned points next
+// to each end become the neighbours' halos.
+template <typename Real, int P>
+struct Exchange {
+    Real* area;           // this warp's shared memory: window [parity][component][32 P], inbox
+    uint64_t (*bar)[2][2];  // warp, side, parity: the neighbour's points are there
+    int H, warp, lane, a0, len;
+    bool left, right, ext_l, ext_r, cluster, by_bar, vec;
+    // what this lane's registers [hb, he) take from a neighbour, and where from
+    // for parity 0 (the neighbour's window in the CTA, or the inbox)
+    int hb, he, hstep;
+    const Real *hu, *hw;
+    ulonglong2 *out_l, *out_r;
+    const ulonglong2 *in_l, *in_r;
+    uint32_t box_l, box_r, bar_l, bar_r;
+    int words;
+
+    // inbox (side, parity) of a warp's area: both components, H values each
+    __device__ __forceinline__ Real* inbox(Real* a, int side, int par) const
+    {
+        return a + 128 * P + (side * 2 + par) * 2 * H;
+    }
+
+    __device__ __forceinline__ void init(const ResExchange& x, const ResWarp* warps, const ResWarp& wd, int g,
+                                         Real* area0, uint64_t (*bars)[2][2])
+    {
+        lane = threadIdx.x & 31;
+        warp = threadIdx.x >> 5;
+        const int nwarp = blockDim.x >> 5;
+        H = x.H;
+        cluster = x.cluster;
+        bar = bars;
+        area = area0 + (size_t)warp * x.warp_values;
+        a0 = wd.lo - wd.start;
+        len = wd.len;
+        left = wd.links & 1;
+        right = wd.links & 2;
+        ext_l = wd.links & 4;
+        ext_r = wd.links & 8;
+        by_bar = cluster || !(ext_l | ext_r);  // (no side is polled in global memory)
+        hb = he = hstep = 0;
+        hu = hw = area;
+        bool v = true;
+        auto clampP = [](int t) { return t < 0 ? 0 : (t > P ? P : t); };
+        const int p0 = lane * P;
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            if (!(side ? right : left)) continue;
+            const int a = side ? a0 + len : a0 - H;  // window positions [a, a + H)
+            const int b = clampP(a - p0), e = clampP(a + H - p0);
+            if (e <= b) continue;
+            hb = b;
+            he = e;
+            const Real* src;
+            if (side ? ext_r : ext_l) {
+                src = inbox(area, side, 0) + (p0 - a);
+                hw = src + H;
+                hstep = 2 * H;
+            } else {
+                // the neighbour's position of this window's position p0
+                const int nb = warp + (side ? 1 : -1);
+                src = area0 + (size_t)nb * x.warp_values + (wd.start + p0 - warps[g + (side ? 1 : -1)].start);
+                hw = src + 32 * P;
+                hstep = 64 * P;
+            }
+            hu = src;
+            constexpr int N = 16 / sizeof(Real);
+            if (b != 0 || e != P || P % N != 0 || ((src - area0) & (N - 1)) != 0 || ((hw - area0) & (N - 1)) != 0)
+                v = false;
+        }
+        vec = __all_sync(kFull, v);
+        // across CTAs: the slots, or in a cluster the neighbours' inboxes and their barriers
+        out_l = out_r = nullptr;
+        in_l = in_r = nullptr;
+        box_l = box_r = bar_l = bar_r = 0;
+        words = H * slot_words<Real>;  // of a slot; parity 1 follows parity 0
+        if (cluster) {
+            if (ext_l) {
+                box_l = cluster_addr(smem_addr(inbox(area0 + (size_t)(nwarp - 1) * x.warp_values, 1, 0)), blockIdx.x - 1);
+                bar_l = cluster_addr(smem_addr(&bars[nwarp - 1][1][0]), blockIdx.x - 1);
+            }
+            if (ext_r) {
+                box_r = cluster_addr(smem_addr(inbox(area0, 0, 0)), blockIdx.x + 1);
+                bar_r = cluster_addr(smem_addr(&bars[0][0][0]), blockIdx.x + 1);
+            }
+        } else {
+            ulonglong2* s = x.xbuf + (int64_t)blockIdx.x * 4 * words;  // [CTA][side][parity]
+            out_l = s;
+            out_r = s + 2 * words;
+            in_l = s - 2 * words;  // the CTA before, its right side
+            in_r = s + 4 * words;  // the CTA after, its left side
+        }
+    }
+
+    // The k-th exchange of the run.  false: a wait ran out (or another warp's
+    // did).  mute: this warp publishes nothing (test hook).
+    __device__ __forceinline__ bool swap(const ResExchange& x, Real (&u)[P], Real (&w)[P], int k, bool mute)
+    {
+        // this warp's window to shared memory, and the H owned
+        // points next to an end that has its neighbour in another CTA onwards
+        const int par = k & 1;
+        const unsigned long long tag = (x.epoch << 32) | (unsigned)(k + 1);
+        Real* const win = area + par * 64 * P;
+        if constexpr (P * sizeof(Real) % 16 == 0) {
+            span::regs_to_smem<Real, P>(win + lane * P, u);
+            span::regs_to_smem<Real, P>(win + 32 * P + lane * P, w);
+        } else {
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+                win[lane * P + i] = u[i];
+                win[32 * P + lane * P + i] = w[i];
+            }
+        }
+        __syncwarp();
+        if (lane < 2 && !mute) {
+            const bool has = lane ? right : left, ext = lane ? ext_r : ext_l;
+            // this warp's points are there, for the neighbour in the CTA; what
+            // the inbox waits for, from the neighbour in the cluster
+            if (has && !ext) mbar_arrive(&bar[lane ? warp + 1 : warp - 1][lane ^ 1][par]);
+            else if (has && cluster)
+                mbar_arrive_expect_tx(&bar[warp][lane][par], (uint32_t)(2 * H * sizeof(Real)));
+        }
+        if (ext_l | ext_r) {
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                if (!(side ? ext_r : ext_l) || mute) continue;
+                const Real* src = win + (side ? a0 + len - H : a0);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int p = lane + 32 * h;
+                    if (p >= H) continue;
+                    const Real a = src[p], b = src[32 * P + p];
+                    if (cluster) {
+                        const uint32_t box = (side ? box_r : box_l) + (uint32_t)((par * 2 * H + p) * sizeof(Real));
+                        const uint32_t nbar = (side ? bar_r : bar_l) + par * 8u;
+                        st_async(box, nbar, a);
+                        st_async(box + (uint32_t)(H * sizeof(Real)), nbar, b);
+                    } else {
+                        ulonglong2* out = (side ? out_r : out_l) + par * words;
+                        if constexpr (sizeof(Real) == 4) {
+                            st_pair(out + p, (unsigned long long)__float_as_uint(a) |
+                                                 ((unsigned long long)__float_as_uint(b) << 32), tag);
+                        } else {
+                            st_pair(out + 2 * p, (unsigned long long)__double_as_longlong(a), tag);
+                            st_pair(out + 2 * p + 1, (unsigned long long)__double_as_longlong(b), tag);
+                        }
+                    }
+                }
+            }
+        }
+        bool ok = true;
+        // (every so many polls: the time limit, and whether another warp gave up)
+        long long t0 = 0;
+        unsigned spins = 0;
+        auto late = [&]() {
+            if ((++spins & 63u) != 0u) return false;
+            const long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            return now - t0 > x.wait_ns || *(volatile int*)&x.err->code != 0;
+        };
+        if (!by_bar) {
+            // both sides are polled together: a poll of L2 is a long round trip
+            bool want[2] = {ext_l, ext_r};
+            for (;;) {
+                unsigned long long y[2][2][4];  // [side][half]: u word, tag, (FP64: w word, tag)
+#pragma unroll
+                for (int side = 0; side < 2; ++side)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int p = lane + 32 * h;
+                        if (!want[side] || p >= H) continue;
+                        const ulonglong2* in = (side ? in_r : in_l) + par * words;
+                        if constexpr (sizeof(Real) == 4) {
+                            ld_pair(in + p, y[side][h][0], y[side][h][1]);
+                        } else {
+                            ld_pair(in + 2 * p, y[side][h][0], y[side][h][1]);
+                            ld_pair(in + 2 * p + 1, y[side][h][2], y[side][h][3]);
+                        }
+                    }
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {
+                    if (!want[side]) continue;
+                    bool all = true;
+                    Real* box = inbox(area, side, par);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int p = lane + 32 * h;
+                        if (p >= H) continue;
+                        if constexpr (sizeof(Real) == 4) {
+                            all = all && y[side][h][1] == tag;
+                            box[p] = __uint_as_float((unsigned)y[side][h][0]);
+                            box[H + p] = __uint_as_float((unsigned)(y[side][h][0] >> 32));
+                        } else {
+                            all = all && y[side][h][1] == tag && y[side][h][3] == tag;
+                            box[p] = __longlong_as_double((long long)y[side][h][0]);
+                            box[H + p] = __longlong_as_double((long long)y[side][h][2]);
+                        }
+                    }
+                    want[side] = !all;
+                }
+                if (__all_sync(kFull, !want[0] && !want[1])) break;
+                if (__any_sync(kFull, late())) {
+                    ok = false;
+                    break;
+                }
+            }
+        }
+        {
+            const uint32_t phase = (uint32_t)(k >> 1) & 1u;
+            if (ok && left && (by_bar || !ext_l))
+                while (!inbox_arrived(&bar[warp][0][par], phase))
+                    if (late()) {
+                        ok = false;
+                        break;
+                    }
+            if (ok && right && (by_bar || !ext_r))
+                while (!inbox_arrived(&bar[warp][1][par], phase))
+                    if (late()) {
+                        ok = false;
+                        break;
+                    }
+            ok = __all_sync(kFull, ok);
+        }
+        if (!ok) return false;
+        __syncwarp();
+        {
+            const Real *su = hu + par * hstep, *sw = hw + par * hstep;
+            if (vec) {
+                if (he > 0) {
+                    if constexpr (P * sizeof(Real) % 16 == 0) {
+                        span::smem_to_regs<Real, P>(su, u);
+                        span::smem_to_regs<Real, P>(sw, w);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < P; ++i)
+                    if (i >= hb && i < he) {
+                        u[i] = su[i];
+                        w[i] = sw[i];
+                    }
+            }
+        }
+        return true;
+    }
+};
+
 template <typename Real, int FORM, int P>
 __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(const __grid_constant__ ResParams<Real> prm)
 {
@@ -322,12 +701,9 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nwarp = blockDim.x >> 5;
-    const int H = prm.H;
     Real* const area0 = reinterpret_cast<Real*>(smem_raw);
-    Real* const area = area0 + (size_t)warp * prm.warp_values;
-    // inbox (side, parity): both components, H values each
-    auto inbox = [&](Real* a, int side, int par) { return a + 128 * P + (side * 2 + par) * 2 * H; };
-    Real* const ring = area + 128 * P + 8 * H;
+    Real* const area = area0 + (size_t)warp * prm.x.warp_values;
+    Real* const ring = area + 128 * P + 8 * prm.x.H;
 
     __shared__ __align__(8) uint64_t s_bar[16][2][2];  // warp, side, parity: the neighbour's points are there
     if (threadIdx.x < 64) mbar_init(&s_bar[0][0][0] + threadIdx.x, 1);
@@ -337,7 +713,7 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
     // a cluster: every inbox exists before anyone writes to it, and (at the
     // end) no CTA leaves while a neighbour may still write to it
     auto cluster_sync = [&]() {
-        if (!prm.cluster) return;
+        if (!prm.x.cluster) return;
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     };
@@ -352,7 +728,6 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
     const ResProb<Real> pb = prm.problems[wd.problem];
     const int nx = (int)pb.nx;
     const int lo = wd.lo, hi = wd.lo + wd.len;
-    const int a0 = lo - wd.start;         // window position of the first owned point
     const int j0 = wd.start + lane * P;   // this lane's first grid point
     const Real c2 = pb.c2, kk = pb.k;
 
@@ -424,52 +799,105 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
         node(nx - 1, pb.fB);
     };
 
-    // ---- probes whose point this warp owns: the first two through rows
+    // ---- probes whose point this warp owns.  fast: one or two, on a lane's first
+    // or last register (the host shifts a window for that): the owner drops the
+    // value (flux: both neighbours) into a small buffer every level.  Else the
+    // first two through rows of all the registers, further ones directly.
     constexpr int RL = kRowLanes<Real>(P);
     const int np = wd.probe_end - wd.probe_begin;
     const ProbeDev<Real>* const probes = prm.probes + wd.probe_begin;
     int pl[2] = {-64, -64}, pr[2] = {0, 0};  // first lane of the row (-64: none), position of the point in it
-    bool slow = np > 2;
+    int fl[2] = {-64, -64};                  // the probe's lane, if it is fast
+    bool at_first[2] = {true, true}, flux[2] = {false, false};
+    bool slow = np > 2, fast = np > 0 && np <= 2;
 #pragma unroll
     for (int q = 0; q < 2; ++q)
         if (q < np) {
             const int pos = (int)probes[q].gidx - wd.start;  // gidx: the grid point
-            const bool flux = probes[q].kind != 0;
-            if (pos < (flux ? 1 : 0) || pos + (flux ? 1 : 0) >= 32 * P) {
+            flux[q] = probes[q].kind != 0;
+            const int o = pos / P, r = pos % P;
+            if (pos < 0 || pos >= 32 * P || (r != 0 && r != P - 1)) fast = false;
+            fl[q] = o;
+            at_first[q] = r == 0;
+            if (pos < (flux[q] ? 1 : 0) || pos + (flux[q] ? 1 : 0) >= 32 * P) {
                 slow = true;  // a node that is not in the window, or a flux next to one
                 continue;
             }
-            const int o = pos / P, r = pos % P;
             pl[q] = r == 0 && o > 0 ? o - 1 : o;
             pr[q] = pos - pl[q] * P;
         }
-    // rows [0, cnt) of the ring hold levels lv0 .. lv0 + cnt - 1
-    auto flush = [&](int64_t lv0, int cnt) {
+    if (fast) pl[0] = pl[1] = -64;
+    // level n into the fast probes' buffers [probe][level mod kFastRing]{value or right, left}
+    auto put_fast = [&](const Real(&x)[P], Real lft, Real rgt, int n) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            Real a, b;
+            if constexpr (P == 1) {
+                a = flux[q] ? rgt : x[0];
+                b = lft;
+            } else {
+                a = at_first[q] ? (flux[q] ? x[1] : x[0]) : (flux[q] ? rgt : x[P - 1]);
+                b = at_first[q] ? lft : x[P - 2];
+            }
+            Real* d = ring + (q * kFastRing + (n & (kFastRing - 1))) * 2;
+            st_shared_if(lane == fl[q], d, a, b);
+            if (np < 2) break;
+        }
+    };
+    // (the writing out reads them every few levels: kept in shared memory)
+    __shared__ ProbeDev<Real> s_probe[16][2];
+    if (lane < 2 && lane < np) s_probe[warp][lane] = probes[lane];
+    __syncwarp();
+    // row n mod kRing holds level n; levels from `first` on are not written out yet
+    int64_t first = 0;
+    auto flush = [&](int64_t end) {
         __syncwarp();
+        const int64_t n = first + lane;
 #pragma unroll
         for (int q = 0; q < 2; ++q)
             if (pl[q] >= 0) {
-                const ProbeDev<Real> p = probes[q];
-                const Real* row = ring + (q * kRing + lane) * RL * P + pr[q];
-                if (lane < cnt && lv0 + lane <= p.nmax) {
+                const ProbeDev<Real>& p = s_probe[warp][q];
+                const Real* row = ring + (q * kRing + (int)(n & (kRing - 1))) * RL * P + pr[q];
+                if (n < end && n <= p.nmax) {
                     const Real val = p.kind == 0 ? row[0] : rsub(row[1], row[-1]);
-                    p.out[(lv0 + lane) * p.stride] = rmul(val, p.scale);
+                    p.out[n * p.stride] = rmul(val, p.scale);
                 }
             }
+        if (fast) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (q < np) {
+                    const ProbeDev<Real>& p = s_probe[warp][q];
+                    const Real* d = ring + (q * kFastRing + (int)(n & (kFastRing - 1))) * 2;
+                    if (n < end && n <= p.nmax) p.out[n * p.stride] = rmul(flux[q] ? rsub(d[0], d[1]) : d[0], p.scale);
+                }
+        }
+        first = end;
         __syncwarp();
     };
-    // level n of the window into row s; further probes directly
-    auto put_rows = [&](const Real(&x)[P], int s, int64_t n) {
+    // level n of the window into its row; further probes directly
+    auto put_rows = [&](const Real(&x)[P], int n) {
+        const int s = n & (kRing - 1);
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int l = lane - pl[q];
-            if (l >= 0 && l < RL) {
-                Real* row = ring + ((q * kRing + s) * RL + l) * P;
-                if constexpr (P * sizeof(Real) % 16 == 0) span::regs_to_smem<Real, P>(row, x);
-                else
+            Real* row = ring + ((q * kRing + s) * RL + l) * P;
+            const bool on = l >= 0 && l < RL && pl[q] >= 0;
+            if constexpr (P % 16 == 0 && sizeof(Real) == 4) {
 #pragma unroll
-                    for (int i = 0; i < P; ++i) row[i] = x[i];
+                for (int i = 0; i < P; i += 16) {
+                    float y[16];
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) y[q] = (float)x[i + q];
+                    st_shared_if16(on, reinterpret_cast<const float*>(row + i), y);
+                }
+            } else if constexpr (P % 2 == 0) {
+#pragma unroll
+                for (int i = 0; i < P; i += 2) st_shared_if(on, row + i, x[i], x[i + 1]);
+            } else {
+                if (on) row[0] = x[0];
             }
+            if (np < 2) break;
         }
         if (slow) {
             Real lf = __shfl_up_sync(kFull, x[P - 1], 1);
@@ -496,10 +924,13 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
             }
         }
     };
-    // the pair of level n of the owned points (a node outside the window: from its samples)
-    auto store_pair = [&](Real* d0, Real* d1, int64_t n) {
-        if (d0) store_owned<Real, P>(d0, u, j0, lo, hi);
-        if (d1) store_owned<Real, P>(d1, w, j0, lo, hi);
+    // the pair of level n of the owned points (a node outside the window: from
+    // its samples); sm: room for one component
+    const int w0 = spec == kNodeLeft ? 0 : lo - wd.start;            // owned window positions [w0, w1)
+    const int w1 = hi - wd.start - (spec == kNodeRight ? 1 : 0);
+    auto store_pair = [&](Real* d0, Real* d1, int64_t n, Real* sm) {
+        if (d0) store_owned<Real, P>(d0 + wd.start, u, sm, lane, w0, w1 - w0);
+        if (d1) store_owned<Real, P>(d1 + wd.start, w, sm, lane, w0, w1 - w0);
         if ((spec == kNodeLeft && lane == 0) || (spec == kNodeRight && lane == 31)) {
             const Real* f = spec == kNodeLeft ? pb.fA : pb.fB;
             const int j = spec == kNodeLeft ? 0 : nx - 1;
@@ -509,256 +940,70 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
         }
     };
 
-    const bool left = wd.links & 1, right = wd.links & 2;
-    const bool ext_l = wd.links & 4, ext_r = wd.links & 8;
-    // what this lane's registers [hb, he) take from a neighbour after a chunk
-    // (the window's halo: H points on a side), and where from, for parity 0:
-    // the neighbour's window in the same CTA, or the inbox
-    int hb = 0, he = 0;
-    const Real *hu = area, *hw = area;
-    int hstep = 0;  // to the same place for parity 1
-    bool vec = true;
-    {
-        auto clampP = [](int x) { return x < 0 ? 0 : (x > P ? P : x); };
-        const int p0 = lane * P;
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-            if (!(side ? right : left)) continue;
-            const int a = side ? a0 + wd.len : a0 - H;  // window positions [a, a + H)
-            const int b = clampP(a - p0), e = clampP(a + H - p0);
-            if (e <= b) continue;
-            hb = b;
-            he = e;
-            const Real* src;
-            if (side ? ext_r : ext_l) {
-                src = inbox(area, side, 0) + (p0 - a);
-                hw = src + H;
-                hstep = 2 * H;
-            } else {
-                // the neighbour's position of this window's position p0
-                const int nb = warp + (side ? 1 : -1);
-                const ResWarp nw = prm.warps[g + (side ? 1 : -1)];
-                src = area0 + (size_t)nb * prm.warp_values + (wd.start + p0 - nw.start);
-                hw = src + 32 * P;
-                hstep = 64 * P;
-            }
-            hu = src;
-            constexpr int N = 16 / sizeof(Real);
-            if (b != 0 || e != P || P % N != 0 || ((src - area0) & (N - 1)) != 0 || ((hw - area0) & (N - 1)) != 0)
-                vec = false;
-        }
-    }
-    vec = __all_sync(kFull, vec);
-    // exchange across CTAs: the slots, or in a cluster the neighbours' inboxes and their barriers
-    ulonglong2 *out_l = nullptr, *out_r = nullptr;
-    const ulonglong2 *in_l = nullptr, *in_r = nullptr;
-    uint32_t box_l = 0, box_r = 0, bar_l = 0, bar_r = 0;
-    const bool by_bar = prm.cluster || !(ext_l | ext_r);  // (no side is polled in global memory)
-    const int words = H * slot_words<Real>;  // of a slot; parity 1 follows parity 0
-    if (prm.cluster) {
-        if (ext_l) {
-            box_l = cluster_addr(smem_addr(inbox(area0 + (size_t)(nwarp - 1) * prm.warp_values, 1, 0)), blockIdx.x - 1);
-            bar_l = cluster_addr(smem_addr(&s_bar[nwarp - 1][1][0]), blockIdx.x - 1);
-        }
-        if (ext_r) {
-            box_r = cluster_addr(smem_addr(inbox(area0, 0, 0)), blockIdx.x + 1);
-            bar_r = cluster_addr(smem_addr(&s_bar[0][0][0]), blockIdx.x + 1);
-        }
-    } else {
-        ulonglong2* x = prm.xbuf + (int64_t)blockIdx.x * 4 * words;  // [CTA][side][parity]
-        out_l = x;
-        out_r = x + 2 * words;
-        in_l = x - 2 * words;  // the CTA before, its right side
-        in_r = x + 4 * words;  // the CTA after, its left side
-    }
+    Exchange<Real, P> ex;
+    ex.init(prm.x, prm.warps, wd, g, area0, s_bar);
     bool ok = true;
+    int kept = 0, part_left = 0;  // states kept so far, steps to the next one
+    const int probe_levels = fast ? kFastRing : kRing;
     const int Tn = (int)prm.T;
     for (int k = 0; k < prm.nchunks; ++k) {
         const int64_t n0 = (int64_t)k * prm.S;
         const int steps = Tn - n0 < prm.S ? (int)(Tn - n0) : prm.S;
-        auto patch = [&](Real(&x)[P], Real(&y)[P], const Real(&xo)[P], int s) { patch_all(x, y, xo, n0 + s); };
-        auto advance = [&](auto&& rec) {
-            switch (spec) {
-                case kPlain:
-                    run_steps<Real, FORM, P, kPlain>(u, w, c2, kk, (int)n0, steps, mine, st, rec, patch);
-                    break;
-                case kNodeLeft:
-                    run_steps<Real, FORM, P, kNodeLeft>(u, w, c2, kk, (int)n0, steps, mine, st, rec, patch);
-                    break;
-                case kNodeRight:
-                    run_steps<Real, FORM, P, kNodeRight>(u, w, c2, kk, (int)n0, steps, mine, st, rec, patch);
-                    break;
-                case kSource:
-                    run_steps<Real, FORM, P, kSource>(u, w, c2, kk, (int)n0, steps, mine, st, rec, patch);
-                    break;
-                default:
-                    run_steps<Real, FORM, P, kAny>(u, w, c2, kk, (int)n0, steps, mine, st, rec, patch);
+        // (with kept states: a state after every part of ck_steps steps, or of
+        // ck_split and ck_steps - ck_split in turn; with probes: the levels up to
+        // the end of their buffer)
+        for (int d0 = 0; d0 < steps;) {
+            const int64_t b0 = n0 + d0;
+            int n = steps - d0;
+            if (prm.ck0) {
+                if (part_left == 0)
+                    part_left = prm.ck_split == 0 ? prm.ck_steps : (kept & 1 ? prm.ck_steps - prm.ck_split : prm.ck_split);
+                n = n < part_left ? n : part_left;
             }
-        };
-        if (np == 0) {
-            advance([](const Real(&)[P], int) {});
-        } else {
-            advance([&](const Real(&x)[P], int s) {
-                put_rows(x, s & (kRing - 1), n0 + s);
-                if ((s & (kRing - 1)) == kRing - 1) flush(n0 + s - (kRing - 1), kRing);
-            });
-            const int rest = steps & (kRing - 1);
-            if (rest) flush(n0 + steps - rest, rest);
-        }
-        // span states kept for the adjoint sweep
-        if (prm.ck0 && (k + 1 < prm.nchunks || prm.ck_last)) {
-            const int64_t o = (int64_t)(k + 1) * prm.ck_stride + pb.base;
-            store_pair(prm.ck0 + o, prm.ck1 + o, n0 + steps);
+            if (np) {
+                const int room = probe_levels - ((int)b0 & (probe_levels - 1));
+                n = n < room ? n : room;
+            }
+            d0 += n;
+            auto patch = [&](Real(&x)[P], Real(&y)[P], const Real(&xo)[P], int s) { patch_all(x, y, xo, b0 + s); };
+            auto advance = [&](auto&& rec) {
+                switch (spec) {
+                    case kPlain:
+                        run_steps<Real, FORM, P, kPlain>(u, w, c2, kk, (int)b0, n, mine, st, rec, patch);
+                        break;
+                    case kNodeLeft:
+                        run_steps<Real, FORM, P, kNodeLeft>(u, w, c2, kk, (int)b0, n, mine, st, rec, patch);
+                        break;
+                    case kNodeRight:
+                        run_steps<Real, FORM, P, kNodeRight>(u, w, c2, kk, (int)b0, n, mine, st, rec, patch);
+                        break;
+                    case kSource:
+                        run_steps<Real, FORM, P, kSource>(u, w, c2, kk, (int)b0, n, mine, st, rec, patch);
+                        break;
+                    default:
+                        run_steps<Real, FORM, P, kAny>(u, w, c2, kk, (int)b0, n, mine, st, rec, patch);
+                }
+            };
+            if (np == 0) {
+                advance([](const Real(&)[P], Real, Real, int) {});
+            } else if (fast) {
+                advance([&](const Real(&x)[P], Real l, Real r, int s) { put_fast(x, l, r, (int)b0 + s); });
+            } else {
+                advance([&](const Real(&x)[P], Real, Real, int s) { put_rows(x, (int)b0 + s); });
+            }
+            if (np && ((int)(b0 + n) & (probe_levels - 1)) == 0) flush(b0 + n);
+            if (prm.ck0 && (part_left -= n) == 0) {
+                const int64_t o = (int64_t)(++kept) * prm.ck_stride + pb.base;
+                // (this exchange's window: free till then)
+                store_pair(prm.ck0 + o, prm.ck1 + o, b0 + n, area + (k & 1) * 64 * P);
+            }
         }
         if (k + 1 == prm.nchunks) break;
 
-        // ---- exchange: this warp's window to shared memory, and the H owned
-        // points next to an end that has its neighbour in another CTA onwards
-        const int par = k & 1;
-        const unsigned long long tag = (prm.epoch << 32) | (unsigned)(k + 1);
-        const bool mute = g == prm.inject_warp && k >= prm.inject_chunk;  // (test hook: stops publishing)
-        Real* const win = area + par * 64 * P;
-        if constexpr (P * sizeof(Real) % 16 == 0) {
-            span::regs_to_smem<Real, P>(win + lane * P, u);
-            span::regs_to_smem<Real, P>(win + 32 * P + lane * P, w);
-        } else {
-#pragma unroll
-            for (int i = 0; i < P; ++i) {
-                win[lane * P + i] = u[i];
-                win[32 * P + lane * P + i] = w[i];
-            }
-        }
-        __syncwarp();
-        if (lane < 2 && !mute) {
-            const bool has = lane ? right : left, ext = lane ? ext_r : ext_l;
-            // this warp's points are there, for the neighbour in the CTA; what
-            // the inbox waits for, from the neighbour in the cluster
-            if (has && !ext) mbar_arrive(&s_bar[lane ? warp + 1 : warp - 1][lane ^ 1][par]);
-            else if (has && prm.cluster)
-                mbar_arrive_expect_tx(&s_bar[warp][lane][par], (uint32_t)(2 * H * sizeof(Real)));
-        }
-        if (ext_l | ext_r) {
-#pragma unroll
-            for (int side = 0; side < 2; ++side) {
-                if (!(side ? ext_r : ext_l) || mute) continue;
-                const Real* src = win + (side ? a0 + wd.len - H : a0);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int p = lane + 32 * h;
-                    if (p >= H) continue;
-                    const Real a = src[p], b = src[32 * P + p];
-                    if (prm.cluster) {
-                        const uint32_t box = (side ? box_r : box_l) + (uint32_t)((par * 2 * H + p) * sizeof(Real));
-                        const uint32_t bar = (side ? bar_r : bar_l) + par * 8u;
-                        st_async(box, bar, a);
-                        st_async(box + (uint32_t)(H * sizeof(Real)), bar, b);
-                    } else {
-                        ulonglong2* out = (side ? out_r : out_l) + par * words;
-                        if constexpr (sizeof(Real) == 4) {
-                            st_pair(out + p, (unsigned long long)__float_as_uint(a) |
-                                                 ((unsigned long long)__float_as_uint(b) << 32), tag);
-                        } else {
-                            st_pair(out + 2 * p, (unsigned long long)__double_as_longlong(a), tag);
-                            st_pair(out + 2 * p + 1, (unsigned long long)__double_as_longlong(b), tag);
-                        }
-                    }
-                }
-            }
-        }
-        // (every so many polls: the time limit, and whether another warp gave up)
-        long long t0 = 0;
-        unsigned spins = 0;
-        auto late = [&]() {
-            if ((++spins & 63u) != 0u) return false;
-            const long long now = global_ns();
-            if (t0 == 0) t0 = now;
-            return now - t0 > prm.wait_ns || *(volatile int*)&prm.err->code != 0;
-        };
-        if (!by_bar) {
-            // both sides are polled together: a poll of L2 is a long round trip
-            bool want[2] = {ext_l, ext_r};
-            for (;;) {
-                unsigned long long x[2][2][4];  // [side][half]: u word, tag, (FP64: w word, tag)
-#pragma unroll
-                for (int side = 0; side < 2; ++side)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int p = lane + 32 * h;
-                        if (!want[side] || p >= H) continue;
-                        const ulonglong2* in = (side ? in_r : in_l) + par * words;
-                        if constexpr (sizeof(Real) == 4) {
-                            ld_pair(in + p, x[side][h][0], x[side][h][1]);
-                        } else {
-                            ld_pair(in + 2 * p, x[side][h][0], x[side][h][1]);
-                            ld_pair(in + 2 * p + 1, x[side][h][2], x[side][h][3]);
-                        }
-                    }
-#pragma unroll
-                for (int side = 0; side < 2; ++side) {
-                    if (!want[side]) continue;
-                    bool all = true;
-                    Real* box = inbox(area, side, par);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int p = lane + 32 * h;
-                        if (p >= H) continue;
-                        if constexpr (sizeof(Real) == 4) {
-                            all = all && x[side][h][1] == tag;
-                            box[p] = __uint_as_float((unsigned)x[side][h][0]);
-                            box[H + p] = __uint_as_float((unsigned)(x[side][h][0] >> 32));
-                        } else {
-                            all = all && x[side][h][1] == tag && x[side][h][3] == tag;
-                            box[p] = __longlong_as_double((long long)x[side][h][0]);
-                            box[H + p] = __longlong_as_double((long long)x[side][h][2]);
-                        }
-                    }
-                    want[side] = !all;
-                }
-                if (__all_sync(kFull, !want[0] && !want[1])) break;
-                if (__any_sync(kFull, late())) {
-                    ok = false;
-                    break;
-                }
-            }
-        }
-        {
-            const uint32_t phase = (uint32_t)(k >> 1) & 1u;
-            if (ok && left && (by_bar || !ext_l))
-                while (!inbox_arrived(&s_bar[warp][0][par], phase))
-                    if (late()) {
-                        ok = false;
-                        break;
-                    }
-            if (ok && right && (by_bar || !ext_r))
-                while (!inbox_arrived(&s_bar[warp][1][par], phase))
-                    if (late()) {
-                        ok = false;
-                        break;
-                    }
-            ok = __all_sync(kFull, ok);
-        }
+        ok = ex.swap(prm.x, u, w, k, g == prm.inject_warp && k >= prm.inject_chunk);
         if (!ok) {
-            latch_error(prm.err, kDevTimeoutFlag, g, k, 0);
+            latch_error(prm.x.err, kDevTimeoutFlag, g, k, 0);
             break;
-        }
-        __syncwarp();
-        {
-            const Real *su = hu + par * hstep, *sw = hw + par * hstep;
-            if (vec) {
-                if (he > 0) {
-                    if constexpr (P * sizeof(Real) % 16 == 0) {
-                        span::smem_to_regs<Real, P>(su, u);
-                        span::smem_to_regs<Real, P>(sw, w);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < P; ++i)
-                    if (i >= hb && i < he) {
-                        u[i] = su[i];
-                        w[i] = sw[i];
-                    }
-            }
         }
     }
     if (!ok) {
@@ -768,10 +1013,18 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
 
     // ---- level T: probes and the state pair
     if (np > 0) {
-        put_rows(u, 0, prm.T);
-        flush(prm.T, 1);
+        if (fast) {
+            Real l = __shfl_up_sync(kFull, u[P - 1], 1), r = __shfl_down_sync(kFull, u[0], 1);
+            if (spec == kNodeLeft && lane == 0) l = node_sample(pb.fA, prm.T);
+            if (spec == kNodeRight && lane == 31) r = node_sample(pb.fB, prm.T);
+            put_fast(u, l, r, (int)prm.T);
+        } else {
+            put_rows(u, (int)prm.T);
+        }
+        flush(prm.T + 1);
     }
-    store_pair(prm.out0 ? prm.out0 + pb.off : nullptr, prm.out1 ? prm.out1 + pb.off : nullptr, prm.T);
+    store_pair(prm.out0 ? prm.out0 + pb.off : nullptr, prm.out1 ? prm.out1 + pb.off : nullptr, prm.T,
+               area + ((prm.nchunks - 1) & 1) * 64 * P);
     cluster_sync();
 }
 

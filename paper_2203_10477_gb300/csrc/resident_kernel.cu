@@ -94,29 +94,39 @@ void configure(cudaLaunchConfig_t* c, cudaLaunchAttribute* at, int grid, int thr
 
 }  // namespace
 
-cudaError_t res_clusters(int dtype, int form, int P, int grid, int threads, size_t smem, int* clusters)
+cudaError_t res_kernel_clusters(const void* fn, int grid, int threads, size_t smem, int* clusters)
 {
     *clusters = 0;
-    const Entry* e = find(dtype, form, P);
-    if (!e) return cudaSuccess;
-    cudaError_t st = cudaFuncSetAttribute(e->fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t st = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (st != cudaSuccess) return st;
     cudaLaunchConfig_t c;
     cudaLaunchAttribute at;
     configure(&c, &at, grid, threads, smem, true, nullptr);
-    return cudaOccupancyMaxActiveClusters(clusters, e->fn, &c);
+    return cudaOccupancyMaxActiveClusters(clusters, fn, &c);
+}
+
+cudaError_t res_launch_kernel(const void* fn, const void* params, int grid, int threads, size_t smem, bool cluster,
+                              cudaStream_t s)
+{
+    void* args[] = {const_cast<void*>(params)};
+    cudaLaunchConfig_t c;
+    cudaLaunchAttribute at;
+    configure(&c, &at, grid, threads, smem, cluster, s);
+    return cudaLaunchKernelExC(&c, fn, args);
+}
+
+cudaError_t res_clusters(int dtype, int form, int P, int grid, int threads, size_t smem, int* clusters)
+{
+    *clusters = 0;
+    const Entry* e = find(dtype, form, P);
+    return e ? res_kernel_clusters(e->fn, grid, threads, smem, clusters) : cudaSuccess;
 }
 
 cudaError_t res_launch(int dtype, int form, int P, const void* params, int grid, int threads, size_t smem,
                        bool cluster, cudaStream_t s)
 {
     const Entry* e = find(dtype, form, P);
-    if (!e) return cudaErrorInvalidValue;
-    void* args[] = {const_cast<void*>(params)};
-    cudaLaunchConfig_t c;
-    cudaLaunchAttribute at;
-    configure(&c, &at, grid, threads, smem, cluster, s);
-    return cudaLaunchKernelExC(&c, e->fn, args);
+    return e ? res_launch_kernel(e->fn, params, grid, threads, smem, cluster, s) : cudaErrorInvalidValue;
 }
 
 }  // namespace rswr

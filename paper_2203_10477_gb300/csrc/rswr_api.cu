@@ -82,7 +82,8 @@ rswr_status validate(const rswr_problem& q)
 struct ResPlan {
     int P = 0, S = 0, H = 0;   // points per lane, steps per exchange, halo
     int nw = 0, per_cta = 0, grid = 0;
-    bool slack = false;        // windows leave room to put a source on a first register
+    int own = 0;               // points of a piece at most
+    bool slack = false;        // windows leave room to put a source or probe on an end register
     bool linked = false;       // some problem has more than one warp
     bool cluster = false;      // the grid is one thread-block cluster
     double cost = 0.0;         // model: ns per step
@@ -824,7 +825,7 @@ int res_own(int P, int H, bool slack) { return 32 * P - 2 * H - (slack ? P - 1 :
 // grid size (P 4 .. 32, H 8 .. 62, 1001 to 2^20 points): the longer of one
 // step's chain and of the work of the warps that share an SM, plus an exchange
 // every S steps (measured 0.8 us inside a cluster, 1.2 us through L2).
-double res_cost(int dtype, int P, int S, int warps_per_sm, bool linked, bool cluster)
+double res_cost(int dtype, int P, int S, int warps_per_sm, bool linked, bool cluster, int probes)
 {
     const double clk = 1.0 / 1.92;  // ns
     double step;
@@ -832,13 +833,15 @@ double res_cost(int dtype, int P, int S, int warps_per_sm, bool linked, bool clu
         step = clk * std::max(192.0 * P, 48.0 * P * warps_per_sm) + 12.0;
     else
         step = clk * std::max({60.0, 8.6 * P, ((warps_per_sm + 3) / 4) * (4.3 * P + 10.0)});
+    // probes: on end registers (1), through rows of registers (2)
+    if (dtype == kF32) step += probes == 0 ? 0.0 : (probes == 1 ? 25.0 : 50.0 + 6.0 * P);
     return step + (linked ? (cluster ? 800.0 : 1200.0) / S : 0.0);
 }
 
 // The best cut with P points per lane (P = 0: over all compiled P); false when
 // the grid does not fit on the GPU at once.  An exchange follows every m spans
 // of S steps, H = m S halo points wide (the Theorem's bound for the windows).
-bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, ResPlan* best)
+bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, bool kept, ResPlan* best)
 {
     static const int Pf[] = {4, 8, 16, 32}, Pd[] = {1, 2, 4, 8, 12, 16};
     const int* Ps = e->dtype == kF64 ? Pd : Pf;
@@ -854,8 +857,9 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources,
             r.P = P;
             r.S = H;
             r.H = H;
-            r.slack = sources && res_own(P, H, true) >= 2 * H + 2;
-            const int own = res_own(P, H, r.slack);
+            r.slack = (sources || probes) && res_own(P, H, true) >= 2 * H + 2;
+            // (kept states want pieces on multiples of four points: 16-byte stores)
+            const int own = r.own = res_own(P, H, r.slack) - (kept ? 4 : 0);
             if (own < 4) break;
             int64_t nw = 0;
             bool fits = true;
@@ -880,7 +884,7 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources,
                 continue;
             }
             if ((int64_t)occ * e->num_sms < r.grid) continue;
-            r.cost = res_cost(e->dtype, P, H, (int)(ctas * r.per_cta), r.linked, false);
+            r.cost = res_cost(e->dtype, P, H, (int)(ctas * r.per_cta), r.linked, false, probes ? (r.slack ? 1 : 2) : 0);
             if (!found || r.cost < best->cost) {
                 *best = r;
                 found = true;
@@ -902,7 +906,7 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources,
                 c.cluster = true;
                 c.per_cta = per_cta;
                 c.grid = grid;
-                c.cost = res_cost(e->dtype, P, H, per_cta, true, true);
+                c.cost = res_cost(e->dtype, P, H, per_cta, true, true, probes ? (r.slack ? 1 : 2) : 0);
                 if (c.cost < best->cost) *best = c;
             }
         }
@@ -911,37 +915,99 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources,
 }
 
 // (remembered per engine: its problems never change)
-bool res_choose(Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, ResPlan* best)
+bool res_choose(Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, bool kept, ResPlan* best)
 {
-    const std::vector<int> key{want_P, S, max_spans, sources, probes, e->inject_tile >= 0};
+    const std::vector<int> key{want_P, S, max_spans, sources, probes, kept, e->inject_tile >= 0};
     auto it = e->res_plans.find(key);
     if (it == e->res_plans.end()) {
         ResPlan r;
-        if (!res_search(e, want_P, S, max_spans, sources, probes, &r)) r.nw = 0;
+        if (!res_search(e, want_P, S, max_spans, sources, probes, kept, &r)) r.nw = 0;
         it = e->res_plans.emplace(key, r).first;
     }
     *best = it->second;
     return best->nw > 0;
 }
 
-// Span states a resident run keeps for the adjoint sweep.
+// States a resident run keeps for the adjoint sweep.
 struct ResKeep {
     void* ck0;
     void* ck1;
-    int64_t stride;              // elements between the states of two chunks
+    int64_t stride;              // elements between two kept states
+    int steps, split;            // ResParams::ck_steps, ck_split
     const int64_t* base;         // per problem: its first point in a state
-    bool last;
 };
+
+// The pieces of a problem of nx points cut into n: piece i starts here, on a
+// multiple of `unit`.
+int64_t res_piece(int64_t nx, int64_t n, int64_t i, int64_t unit) { return i >= n ? nx : i * nx / n / unit * unit; }
+
+// Appends the pieces of problem p as warps, per_cta of them to a CTA (windows
+// start one halo left of the piece).
+void res_add_pieces(std::vector<ResWarp>* warps, int p, int64_t nx, int64_t n, int64_t unit, int H, int per_cta)
+{
+    for (int64_t i = 0; i < n; ++i) {
+        ResWarp w{};
+        w.problem = p;
+        w.lo = (int32_t)res_piece(nx, n, i, unit);
+        w.len = (int32_t)(res_piece(nx, n, i + 1, unit) - w.lo);
+        w.start = w.lo - H;
+        if (i > 0) w.links |= 1;
+        if (i + 1 < n) w.links |= 2;
+        const int64_t g = (int64_t)warps->size();
+        if ((w.links & 1) && g % per_cta == 0) w.links |= 4;
+        if ((w.links & 2) && g % per_cta == per_cta - 1) w.links |= 8;
+        warps->push_back(w);
+    }
+}
+
+// Exchange slots of a launch (zeroed once: every launch has its own tag).
+rswr_status res_slots(Engine* e, size_t bytes, cudaStream_t s)
+{
+    if (bytes <= e->xbuf_cap) return RSWR_OK;
+    RSWR_CUDA(cudaStreamSynchronize(s));
+    cudaFree(e->d_xbuf);
+    e->d_xbuf = nullptr;
+    e->xbuf_cap = 0;
+    if (cudaMalloc(&e->d_xbuf, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(RSWR_ENOMEM, "halo exchange slots");
+    }
+    e->xbuf_cap = bytes;
+    RSWR_CUDA(cudaMemsetAsync(e->d_xbuf, 0, bytes, s));
+    e->res_epoch = 0;
+    return RSWR_OK;
+}
+
+ResExchange res_exchange(Engine* e, int H, int values, bool cluster)
+{
+    ResExchange x{};
+    x.xbuf = static_cast<ulonglong2*>(e->d_xbuf);
+    x.epoch = ++e->res_epoch;
+    x.err = e->d_err;
+    x.wait_ns = (long long)(e->wait_s * 1e9);
+    x.H = H;
+    x.warp_values = values;
+    x.cluster = cluster;
+    return x;
+}
+
+// (tags of launches would repeat in a replayed graph)
+rswr_status res_no_capture(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    RSWR_CUDA(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+        return fail(RSWR_ECUDA, "runs cannot be captured: every launch carries its own exchange tag");
+    return RSWR_OK;
+}
 
 // One resident run: tables, one upload (skipped when the device holds the same
 // bytes already), one cooperative launch.
 template <typename Real>
 rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep* keep, cudaStream_t s)
 {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    RSWR_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (cap != cudaStreamCaptureStatusNone)
-        return fail(RSWR_ECUDA, "runs cannot be captured: every launch carries its own exchange tag");
+    rswr_status st = res_no_capture(s);
+    if (st != RSWR_OK) return st;
     const size_t np = e->probs.size();
     const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
     if (r.user_src && !e->usrc.empty() && e->usrc_pitch < r.T + 1)
@@ -952,7 +1018,7 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     std::vector<ResWarp> warps;
     std::vector<int32_t> first(np + 1);
     warps.reserve(rp.nw);
-    const int own = res_own(rp.P, rp.H, rp.slack);
+    const int own = rp.own;
     for (size_t p = 0; p < np; ++p) {
         const ProbHost& ph = e->probs[p];
         ResProb<Real>& d = probs[p];
@@ -965,26 +1031,48 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
         d.k = sizeof(Real) == 8 ? (Real)ph.k : (Real)ph.kf;
         first[p] = (int32_t)warps.size();
         const int64_t n = (ph.nx + own - 1) / own;
-        // even pieces, starting on multiples of four points (16-byte stores)
-        // where every piece still holds a strip of H points
-        const int64_t unit = n > 1 && ph.nx / n - 4 > rp.H && (ph.nx + n - 1) / n + 4 <= own ? 4 : 1;
-        for (int64_t i = 0; i < n; ++i) {
-            ResWarp w{};
-            const int64_t lo = i * ph.nx / n / unit * unit;
-            const int64_t hi = i + 1 == n ? ph.nx : (i + 1) * ph.nx / n / unit * unit;
-            w.problem = (int32_t)p;
-            w.lo = (int32_t)lo;
-            w.len = (int32_t)(hi - lo);
-            if (i > 0) w.links |= 1;
-            if (i + 1 < n) w.links |= 2;
-            w.start = w.lo - rp.H;
-            const int64_t g = (int64_t)warps.size();
-            if ((w.links & 1) && g % rp.per_cta == 0) w.links |= 4;
-            if ((w.links & 2) && g % rp.per_cta == rp.per_cta - 1) w.links |= 8;
-            warps.push_back(w);
-        }
+        // even pieces on multiples of four points (16-byte stores) where every
+        // piece still holds more points than a halo
+        const int64_t unit = n > 1 && ph.nx / n - 4 > rp.H && (ph.nx + n - 1) / n + 4 <= own + (keep ? 4 : 0) ? 4 : 1;
+        res_add_pieces(&warps, (int)p, ph.nx, n, unit, rp.H, rp.per_cta);
     }
     first[np] = (int32_t)warps.size();
+
+    // probes by grid point, ranges per warp
+    std::vector<ProbeDev<Real>> probes;
+    std::vector<int32_t> prob_of;
+    {
+        std::vector<size_t> order(r.probes.size());
+        for (size_t i = 0; i < order.size(); ++i) order[i] = i;
+        std::sort(order.begin(), order.end(), [&](size_t a, size_t b) {
+            const ProbeReq &x = r.probes[a], &y = r.probes[b];
+            return x.p != y.p ? x.p < y.p : x.j < y.j;
+        });
+        size_t g = 0;
+        for (size_t i = 0; i < order.size(); ++i) {
+            const ProbeReq& q = r.probes[order[i]];
+            const ProbHost& ph = e->probs[q.p];
+            ProbeDev<Real> d{};
+            d.gidx = q.j;
+            d.out = static_cast<Real*>(q.out);
+            d.stride = q.stride;
+            d.nmax = q.nmax;
+            d.kind = q.kind;
+            if (q.scale_is_c2) d.scale = sizeof(Real) == 8 ? (Real)ph.c2 : (Real)ph.c2f;
+            else if (q.kind == 1) d.scale = sizeof(Real) == 8 ? (Real)ph.inv2dx : (Real)ph.inv2dxf;
+            else d.scale = (Real)q.scale;
+            while (g < warps.size() && (warps[g].problem < q.p ||
+                                        (warps[g].problem == q.p && (int64_t)warps[g].lo + warps[g].len <= q.j))) {
+                warps[g].probe_end = (int32_t)i;
+                if (++g < warps.size()) warps[g].probe_begin = (int32_t)i;
+            }
+            probes.push_back(d);
+        }
+        if (!order.empty()) {
+            warps[g].probe_end = (int32_t)order.size();
+            for (++g; g < warps.size(); ++g) warps[g].probe_begin = warps[g].probe_end = (int32_t)order.size();
+        }
+    }
 
     // sources, grouped by warp in the caller's order: those among a piece and
     // the halos it needs
@@ -1024,7 +1112,22 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
             const bool l = w.links & 1, rt = w.links & 2;
             w.spec = 0;
             if (l && rt) {
-                if (n == 0) continue;
+                if (n == 0) {
+                    // one or two probes: on end registers, where a shift within the window does it
+                    const int np_w = w.probe_end - w.probe_begin;
+                    for (int sh = 0; (np_w == 1 || np_w == 2) && sh < rp.P && 2 * rp.H + sh + w.len <= 32 * rp.P; ++sh) {
+                        bool good = true;
+                        for (int32_t i = w.probe_begin; i < w.probe_end; ++i) {
+                            const int r = (int)((probes[i].gidx - (w.start - sh)) % rp.P);
+                            good = good && (r == 0 || r == rp.P - 1);
+                        }
+                        if (good) {
+                            w.start -= sh;
+                            break;
+                        }
+                    }
+                    continue;
+                }
                 const int shift = (int)((((int64_t)w.start - srcs[w.src_begin].j) % rp.P + rp.P) % rp.P);
                 const bool fits = n == 1 && rp.H + shift + w.len + rp.H <= 32 * rp.P;
                 if (fits) w.start -= shift;
@@ -1038,42 +1141,6 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
                 w.start = (int32_t)(e->probs[w.problem].nx - 1 - 32 * rp.P);
                 w.spec = 2;
             }
-        }
-    }
-
-    // probes by grid point, ranges per warp
-    std::vector<ProbeDev<Real>> probes;
-    std::vector<int32_t> prob_of;
-    {
-        std::vector<size_t> order(r.probes.size());
-        for (size_t i = 0; i < order.size(); ++i) order[i] = i;
-        std::sort(order.begin(), order.end(), [&](size_t a, size_t b) {
-            const ProbeReq &x = r.probes[a], &y = r.probes[b];
-            return x.p != y.p ? x.p < y.p : x.j < y.j;
-        });
-        size_t g = 0;
-        for (size_t i = 0; i < order.size(); ++i) {
-            const ProbeReq& q = r.probes[order[i]];
-            const ProbHost& ph = e->probs[q.p];
-            ProbeDev<Real> d{};
-            d.gidx = q.j;
-            d.out = static_cast<Real*>(q.out);
-            d.stride = q.stride;
-            d.nmax = q.nmax;
-            d.kind = q.kind;
-            if (q.scale_is_c2) d.scale = sizeof(Real) == 8 ? (Real)ph.c2 : (Real)ph.c2f;
-            else if (q.kind == 1) d.scale = sizeof(Real) == 8 ? (Real)ph.inv2dx : (Real)ph.inv2dxf;
-            else d.scale = (Real)q.scale;
-            while (g < warps.size() && (warps[g].problem < q.p ||
-                                        (warps[g].problem == q.p && (int64_t)warps[g].lo + warps[g].len <= q.j))) {
-                warps[g].probe_end = (int32_t)i;
-                if (++g < warps.size()) warps[g].probe_begin = (int32_t)i;
-            }
-            probes.push_back(d);
-        }
-        if (!order.empty()) {
-            warps[g].probe_end = (int32_t)order.size();
-            for (++g; g < warps.size(); ++g) warps[g].probe_begin = warps[g].probe_end = (int32_t)order.size();
         }
     }
 
@@ -1099,20 +1166,7 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
         }
         e->res_cap = tab.size();
     }
-    const size_t xb = res_slot_bytes(e->dtype, rp.H) * rp.grid;
-    if (xb > e->xbuf_cap) {
-        RSWR_CUDA(cudaStreamSynchronize(s));
-        cudaFree(e->d_xbuf);
-        e->d_xbuf = nullptr;
-        e->xbuf_cap = 0;
-        if (cudaMalloc(&e->d_xbuf, xb) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(RSWR_ENOMEM, "halo exchange slots");
-        }
-        e->xbuf_cap = xb;
-        RSWR_CUDA(cudaMemsetAsync(e->d_xbuf, 0, xb, s));
-        e->res_epoch = 0;
-    }
+    if ((st = res_slots(e, res_slot_bytes(e->dtype, rp.H) * rp.grid, s)) != RSWR_OK) return st;
     if (tab != e->res_tables) {
         RSWR_CUDA(cudaMemcpyAsync(e->d_res, tab.data(), tab.size(), cudaMemcpyHostToDevice, s));
         e->res_tables = std::move(tab);
@@ -1133,27 +1187,22 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
         prm.ck0 = static_cast<Real*>(keep->ck0);
         prm.ck1 = static_cast<Real*>(keep->ck1);
         prm.ck_stride = keep->stride;
-        prm.ck_last = keep->last;
+        prm.ck_steps = keep->steps;
+        prm.ck_split = keep->split;
     }
     const int64_t steps = r.stop >= 0 ? r.stop : r.T;
     prm.T = steps;
     prm.S = rp.S;
-    prm.H = rp.H;
     prm.nchunks = (int32_t)((steps + rp.S - 1) / rp.S);
     // a flux of level T at a piece's end reads a halo point, which a full chunk
     // uses up: one more exchange before the last level is recorded
     if (!r.probes.empty() && steps % rp.S == 0) prm.nchunks += 1;
     prm.nwarps = (int32_t)warps.size();
-    prm.cluster = rp.cluster;
     prm.inject_warp = e->inject_tile;
     prm.inject_chunk = (int32_t)((int64_t)e->inject_span * e->S / rp.S);
-    prm.xbuf = static_cast<ulonglong2*>(e->d_xbuf);
-    prm.epoch = ++e->res_epoch;
-    prm.err = e->d_err;
-    prm.wait_ns = (long long)(e->wait_s * 1e9);
     int values = 0;
     const size_t smem = res_smem_bytes(e->dtype, rp.P, rp.H, rp.per_cta, r.probes.empty() ? 0 : 2, &values);
-    prm.warp_values = values;
+    prm.x = res_exchange(e, rp.H, values, rp.cluster);
     if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
     RSWR_CUDA(res_launch(e->dtype, e->form, rp.P, &prm, rp.grid, 32 * rp.per_cta, smem, rp.cluster, s));
     if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
@@ -1171,11 +1220,11 @@ rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
     const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
     if (r.mono || r.from_state || r.steps_dev || r.T <= 0 || r.T >= ((int64_t)1 << 31) - 256) return RSWR_OK;
     if (vi.resident) {
-        if (!res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), rp))
+        if (!res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp))
             return fail(RSWR_ENOTSUP, "resident variant: the grid does not fit on the GPU at once");
         *take = true;
     } else if (!e->chosen && e->mode == RSWR_MODE_PERSISTENT && e->inject_tile < 0) {
-        *take = res_choose(e, 0, e->S, kResMaxHalo, sources, !r.probes.empty(), rp);
+        *take = res_choose(e, 0, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp);
     }
     return RSWR_OK;
 }
@@ -1394,6 +1443,107 @@ rswr_status adjoint_g(Engine* e, int64_t T, const int64_t* j_r, const void* wbar
 
 namespace {
 
+// ---- the resident adjoint sweep (resident_adjoint.cu) ---------------------
+
+struct RadjPlan {
+    int v = -1, P = 0, E = 0, H = 0;
+    int span = 0, split = 0;      // steps of a span; > 0: of its first part
+    int nw = 0, per_cta = 0, grid = 0;
+    bool cluster = false;
+    std::vector<int64_t> pieces;  // per problem
+    ResPlan fwd;                  // the forward sweep's cut
+    double cost = 1e300;
+};
+
+// Pieces of a problem: as few as fit the windows, two at least, on multiples of
+// P (a lane then owns all of its points or none, but for the grid's ends).  0:
+// cannot be cut.
+int64_t radj_pieces(int64_t nx, int P, int own, int H)
+{
+    for (int64_t n = std::max<int64_t>(2, (nx + own - 1) / own); n <= nx / (H + 1); ++n) {
+        if (nx / n - P <= H) return 0;
+        if ((nx + n - 1) / n + P <= own) return n;
+    }
+    return 0;
+}
+
+// Whether the gradient takes the resident sweep, and its cut: plans as they were
+// created and plans on a resident variant, when the grid fits on the chip.
+bool radj_choose(Engine* e, int64_t T, RadjPlan* best)
+{
+    const VariantInfo vplan = span_variant_info(e->variant);
+    if (!(vplan.resident || (!e->chosen && e->mode == RSWR_MODE_PERSISTENT)) || e->ck_spacing > 1) return false;
+    if (T < 1 || T >= ((int64_t)1 << 31) - 256) return false;
+    for (int v = 0; v < radj_variants(); ++v) {
+        int dt, form, P, SA, most;
+        radj_info(v, &dt, &form, &P, &SA, &most);
+        if (dt != e->dtype || form != e->form) continue;
+        // FP32 sums dL/da over the spans of the other sweeps (adjoint_full), in
+        // one or two parts of at most SA levels
+        const int span = e->dtype == kF32 ? std::min(e->S, 16) : SA;
+        for (int E = 1; E * span <= 32; ++E) {
+            RadjPlan r;
+            r.v = v;
+            r.P = P;
+            r.span = span;
+            r.split = span > SA ? (span + 1) / 2 : 0;
+            r.E = E;
+            r.H = (E * span + P - 1) / P * P;
+            const int own = 32 * P - 2 * r.H;
+            if (own <= r.H) continue;
+            int64_t nw = 0;
+            for (const ProbHost& ph : e->probs) {
+                const int64_t n = radj_pieces(ph.nx, P, own, r.H);
+                nw = n ? nw + n : -1;
+                if (!n || nw > (int64_t)e->num_sms * most) break;
+                r.pieces.push_back(n);
+            }
+            if (r.pieces.size() != e->probs.size() || nw > (int64_t)e->num_sms * most) continue;
+            r.nw = (int)nw;
+            // one CTA to an SM; up to 16 CTAs as one cluster
+            for (int cl = 0; cl < 2; ++cl) {
+                for (int per = cl ? 4 : (int)((nw + e->num_sms - 1) / e->num_sms); per <= most; per += 4) {
+                    RadjPlan c = r;
+                    c.cluster = cl == 1;
+                    c.per_cta = per;
+                    c.grid = (c.nw + per - 1) / per;
+                    if (cl && c.grid > 16) continue;
+                    // model (ns per level, fitted as res_cost): eight FP64 operations of 64 clocks
+                    // per point and warp; FP32 12 P + 45 issue slots, a chain of two steps
+                    const double clk = 1.0 / 1.92;
+                    const double step =
+                        e->dtype == kF64 ? clk * std::max(512.0 * P, 128.0 * P * per) + 25.0
+                                         : clk * std::max(130.0 + 17.0 * P, ((per + 3) / 4) * (12.0 * P + 45.0));
+                    c.cost = step + (cl ? 800.0 : 1200.0) / c.H;
+                    if (c.cost >= best->cost) break;
+                    int values = 0, fit = 1;
+                    bool ok = false;
+                    const size_t smem = radj_smem_bytes(v, c.H, per, &values);
+                    if (radj_fits(v, smem, &ok) != cudaSuccess || !ok ||
+                        (cl && (radj_clusters(v, c.grid, 32 * per, smem, &fit) != cudaSuccess || fit < 1))) {
+                        cudaGetLastError();
+                        if (!cl) break;
+                        continue;
+                    }
+                    *best = c;
+                    break;
+                }
+            }
+        }
+    }
+    // the forward sweep exchanges every so many spans
+    return best->v >= 0 && res_choose(e, 0, best->span, kResMaxHalo / best->span, false, true, true, &best->fwd);
+}
+
+struct KeepReq;
+
+// adjoint_full on resident warps.  *done = false: the kept states do not fit in
+// half of the free memory (the caller's other sweeps checkpoint sparsely).
+template <typename Real>
+rswr_status adjoint_resident(Engine* e, int64_t T, const int64_t* j_r, const void* fA, const void* fB,
+                             const void* wbar, void* grad, double* grad_a, cudaStream_t s, const KeepReq* keep,
+                             const RadjPlan& rj, bool* done);
+
 // Gradients of <wbar, receiver trace> w.r.t. fA and a with the forward levels
 // recomputed from checkpoints (see adjoint_kernel.cu for the kernel side).
 //   spans of SA steps (SA <= the adjoint variant's shared-memory store and <= S);
@@ -1411,11 +1561,160 @@ struct KeepReq {
 };
 
 template <typename Real>
+rswr_status adjoint_resident(Engine* e, int64_t T, const int64_t* j_r, const void* fA, const void* fB,
+                             const void* wbar, void* grad, double* grad_a, cudaStream_t s, const KeepReq* keep,
+                             const RadjPlan& rj, bool* done)
+{
+    *done = false;
+    const int np = (int)e->probs.size();
+    const size_t es = sizeof(Real);
+    const int64_t nspans = (T + rj.span - 1) / rj.span;
+    const int64_t rest = T - (nspans - 1) * rj.span;  // steps of the last span
+    const int64_t parts = rj.split ? 2 * (nspans - 1) + (rest > rj.split ? 2 : 1) : nspans;
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    std::vector<int64_t> base(np), t0(np), tc(np);
+    int64_t at = 0, nw = 0;
+    for (int p = 0; p < np; ++p) {
+        base[p] = at;
+        at += (e->probs[p].nx + kAlign - 1) / kAlign * kAlign;
+        t0[p] = nw;
+        tc[p] = rj.pieces[p];
+        nw += tc[p];
+    }
+    const size_t arr = up(es * at);
+    const size_t b_states = 2 * arr * (size_t)(parts + 2);
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || b_states > (free_b + e->adj_mem_cap) / 2) {
+        cudaGetLastError();
+        return RSWR_OK;
+    }
+    *done = true;
+    rswr_status st = res_no_capture(s);
+    if (st != RSWR_OK) return st;
+    const size_t b_prob = up(sizeof(ResAdjProb<Real>) * np), b_warp = up(sizeof(ResWarp) * nw);
+    const size_t b_red = up(sizeof(int64_t) * 2 * np + sizeof(double) * np);
+    const size_t b_sums = up(sizeof(double) * nw), b_tmp = up(sizeof(double) * np);
+    const size_t need = b_states + b_prob + b_warp + b_red + b_sums + b_tmp;
+    const Engine::KeptKey key{fA, fB, T, rj.span, -1, rj.v, rj.H, rj.nw, 1, true, arr, need};
+    const bool reuse = !keep && e->kept && e->kept_key == key && need <= e->adj_mem_cap;
+    if (!reuse) e->kept = false;
+    if (need > e->adj_mem_cap) {
+        RSWR_CUDA(cudaStreamSynchronize(s));
+        cudaFree(e->adj_mem);
+        e->adj_mem = nullptr;
+        e->adj_mem_cap = 0;
+        if (cudaMalloc(&e->adj_mem, need) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(RSWR_ENOMEM, "adjoint workspace (" + std::to_string(need) + " bytes)");
+        }
+        e->adj_mem_cap = need;
+    }
+    char* q = static_cast<char*>(e->adj_mem);
+    Real* ck0 = reinterpret_cast<Real*>(q);
+    Real* ck1 = reinterpret_cast<Real*>(q + arr);
+    const int64_t stride = (int64_t)(2 * arr / es);
+    char* d_tab = q + b_states;
+    double* d_sums = reinterpret_cast<double*>(d_tab + b_prob + b_warp + b_red);
+    double* d_tmp = reinterpret_cast<double*>(d_tab + b_prob + b_warp + b_red + b_sums);
+
+    // the forward sweep: the state at the start of every part (a kept run: to the
+    // end, with the receiver trace and the final state)
+    if (!reuse) {
+        RSWR_CUDA(cudaMemsetAsync(ck0, 0, 2 * arr, s));
+        RunReq r;
+        r.fA = fA;
+        r.fB = fB;
+        r.T = T;
+        const ResKeep rk{ck0, ck1, stride, rj.span, rj.split, base.data()};
+        if (keep) {
+            r.out0 = keep->out0;
+            r.out1 = keep->out1;
+            if (keep->recv) r.probes.push_back(ProbeReq{0, keep->j_rec, 0, 1.0, keep->recv, 1, T});
+        } else {
+            r.stop = (nspans - 1) * rj.span + (rj.split && rest > rj.split ? rj.split : 0);
+        }
+        if (keep || r.stop > 0) st = res_run<Real>(e, r, rj.fwd, &rk, s);
+        else RSWR_CUDA(cudaMemsetAsync(e->d_err, 0, sizeof(DevError), s));
+        if (st != RSWR_OK) return st;
+        if (keep) {
+            e->kept = true;
+            e->kept_key = key;
+            return RSWR_OK;
+        }
+    } else {
+        RSWR_CUDA(cudaMemsetAsync(e->d_err, 0, sizeof(DevError), s));
+    }
+
+    // tables: problems, warps, and the reduction's ranges and scales
+    std::vector<unsigned char> tab(b_prob + b_warp + b_red, 0);
+    auto* probs = reinterpret_cast<ResAdjProb<Real>*>(tab.data());
+    std::vector<ResWarp> warps;
+    warps.reserve(nw);
+    auto* red = reinterpret_cast<int64_t*>(tab.data() + b_prob + b_warp);
+    auto* scale = reinterpret_cast<double*>(red + 2 * np);
+    RSWR_CUDA(cudaMemsetAsync(grad, 0, es * (T + 1) * np, s));
+    for (int p = 0; p < np; ++p) {
+        const ProbHost& ph = e->probs[p];
+        ResAdjProb<Real>& d = probs[p];
+        d.base = base[p];
+        d.nx = ph.nx;
+        d.fA = fA ? static_cast<const Real*>(fA) + (int64_t)p * (T + 1) : nullptr;
+        d.fB = fB ? static_cast<const Real*>(fB) + (int64_t)p * (T + 1) : nullptr;
+        d.wbar = static_cast<const Real*>(wbar) + (int64_t)p * (T + 1);
+        d.grad = static_cast<Real*>(grad) + (int64_t)p * (T + 1);
+        d.c2 = es == 8 ? (Real)ph.c2 : (Real)ph.c2f;
+        d.k = es == 8 ? (Real)ph.k : (Real)ph.kf;
+        d.js = j_r[p] > 0 && j_r[p] < ph.nx - 1 ? (int32_t)j_r[p] : -1;
+        red[p] = t0[p];
+        red[np + p] = tc[p];
+        scale[p] = 2.0 * ph.c2 / ph.a;
+        // a receiver on the left Dirichlet node: dL/dfA is wbar itself
+        if (j_r[p] == 0)
+            RSWR_CUDA(cudaMemcpyAsync(d.grad, d.wbar, es * (T + 1), cudaMemcpyDeviceToDevice, s));
+        res_add_pieces(&warps, p, ph.nx, tc[p], rj.P, rj.H, rj.per_cta);
+        warps[t0[p]].start = 0;  // (the left node on the first register)
+    }
+    std::memcpy(tab.data() + b_prob, warps.data(), sizeof(ResWarp) * nw);
+    RSWR_CUDA(cudaMemcpyAsync(d_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, s));
+    if ((st = res_slots(e, res_slot_bytes(e->dtype, rj.H) * rj.grid, s)) != RSWR_OK) return st;
+    int values = 0;
+    const size_t smem = radj_smem_bytes(rj.v, rj.H, rj.per_cta, &values);
+    ResAdjParams<Real> prm{};
+    prm.x = res_exchange(e, rj.H, values, rj.cluster);
+    prm.problems = reinterpret_cast<const ResAdjProb<Real>*>(d_tab);
+    prm.warps = reinterpret_cast<const ResWarp*>(d_tab + b_prob);
+    prm.uck0 = ck0;
+    prm.uck1 = ck1;
+    prm.ck_stride = stride;
+    prm.T = T;
+    prm.sums = d_sums;
+    prm.nspans = (int32_t)nspans;
+    prm.nwarps = (int32_t)nw;
+    prm.span = rj.span;
+    prm.split = rj.split;
+    prm.parts = (int32_t)parts;
+    prm.E = rj.E;
+    RSWR_CUDA(radj_launch(rj.v, &prm, rj.grid, 32 * rj.per_cta, smem, rj.cluster, s));
+    if (grad_a) {
+        const int64_t* d_red = reinterpret_cast<const int64_t*>(d_tab + b_prob + b_warp);
+        RSWR_CUDA(adj_reduce_launch(d_sums, 1, nw, d_red, d_red + np, reinterpret_cast<const double*>(d_red + 2 * np),
+                                    grad_a, np, d_tmp, s));
+    }
+    return RSWR_OK;
+}
+
+template <typename Real>
 rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* fA, const void* fB, const void* wbar,
                          void* grad, double* grad_a, cudaStream_t s, const KeepReq* keep = nullptr)
 {
     const int np = (int)e->probs.size();
     const size_t es = sizeof(Real);
+    RadjPlan rj;
+    if (radj_choose(e, T, &rj)) {
+        bool done = false;
+        rswr_status st = adjoint_resident<Real>(e, T, j_r, fA, fB, wbar, grad, grad_a, s, keep, rj, &done);
+        if (done || st != RSWR_OK) return st;
+    }
     int va = -1;
     for (int v = 0; v < adj_variant_count(); ++v) {
         const VariantInfo vi = adj_variant_info(v);
@@ -1506,14 +1805,6 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
         make_layout(ai.W - 2 * H);
         C = spacing();
     }
-    // With every span state kept, the checkpoint sweep of a grid that fits on
-    // the chip is one resident launch (an exchange per span, every span's end
-    // written out): on small grids the ticketed sweep is paced by one tile's
-    // chain per span.
-    ResPlan rp;
-    const bool res_sweep = C == 1 && nspans > 0 && T < ((int64_t)1 << 31) - 256 &&
-                           (vplan.resident || (!e->chosen && e->mode == RSWR_MODE_PERSISTENT)) &&
-                           res_choose(e, 0, SA, 1, false, keep && keep->recv, &rp);
     if (keep && C != 1) return fail(RSWR_ENOMEM, "the span states of this run do not fit in device memory");
     const int64_t nck = std::max<int64_t>(1, (nspans + C - 1) / C);
     const int64_t nstates = nck + C + 4;  // checkpoints | segment | forward work pair | adjoint pair
@@ -1530,7 +1821,7 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
     const size_t need = b_states + b_partial + b_tiles + b_prob + b_probes + b_red + b_done + b_rtmp;
     // the span states of an earlier sweep with the same inputs and layout are
     // still in the workspace: the forward sweep can be skipped
-    const Engine::KeptKey key{fA, fB, T, SA, res_sweep ? -1 : vf, va, core_f, core_a, C, use_ws, arr, need};
+    const Engine::KeptKey key{fA, fB, T, SA, vf, va, core_f, core_a, C, use_ws, arr, need};
     const bool reuse = !keep && e->kept && e->kept_key == key && need <= e->adj_mem_cap;
     if (!reuse) e->kept = false;
     if (need > e->adj_mem_cap) {
@@ -1692,24 +1983,7 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
     if (!reuse) {
     RSWR_CUDA(cudaMemsetAsync(state0(CK0), 0, 2 * arr, s));
     RSWR_CUDA(set_boundary_launch(e->dtype, e->form, state0(CK0), state1(CK0), d_pu, np, s));
-    if (res_sweep) {
-        RunReq r;
-        r.fA = fA;
-        r.fB = fB;
-        r.T = T;
-        const ResKeep rk{state0(CK0), state1(CK0), (int64_t)(2 * arr / es), base.data(), !keep};
-        if (keep) {
-            r.out0 = keep->out0;
-            r.out1 = keep->out1;
-            if (keep->recv) r.probes.push_back(ProbeReq{0, keep->j_rec, 0, 1.0, keep->recv, 1, T});
-        } else {
-            r.stop = last_ck_span * SA;
-        }
-        if (keep || last_ck_span > 0) {
-            rswr_status st = res_run<Real>(e, r, rp, &rk, s);
-            if (st != RSWR_OK) return st;
-        }
-    } else if (C == 1 && last_ck_span > 0) {
+    if (C == 1 && last_ck_span > 0) {
         // every span state is kept: the whole sweep is one persistent launch in
         // which span k reads state k and writes state k + 1 (neighbour flags as in
         // rswr_run; the states are distinct arrays, so only read-after-write waits)
@@ -1742,7 +2016,6 @@ rswr_status adjoint_full(Engine* e, int64_t T, const int64_t* j_r, const void* f
         e->kept_key = key;
     }
 
-    if (keep && res_sweep) return RSWR_OK;  // (receiver and final state written by the resident run)
     if (keep) {
         // a kept forward run: the last span into the work pair, the receiver's
         // last level, the final state pair

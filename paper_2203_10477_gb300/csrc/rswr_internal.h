@@ -217,8 +217,21 @@ struct ResSrc {
     int32_t j, pad_;
 };
 
+// What an exchange between resident warps needs.
+struct ResExchange {
+    ulonglong2* xbuf;          // slots [CTA][side][parity][H * words]
+    unsigned long long epoch;  // of this launch, part of the slots' tags
+    DevError* err;
+    long long wait_ns;
+    int32_t H;                 // halo of a window
+    int32_t warp_values;       // shared-memory values of one warp
+    int32_t cluster;           // 1: the grid is one thread-block cluster
+    int32_t pad_;
+};
+
 template <typename Real>
 struct ResParams {
+    ResExchange x;
     const ResProb<Real>* problems;
     const ResWarp* warps;
     const ProbeDev<Real>* probes;  // gidx: the grid point
@@ -227,23 +240,47 @@ struct ResParams {
     const Real* in1;
     Real* out0;                    // packed final state
     Real* out1;
-    Real* ck0;                     // kept span states: chunk k ends in ck + (k + 1) * ck_stride (null: none)
+    Real* ck0;                     // kept states: the i-th after level 0 at ck + i * ck_stride (null: none)
     Real* ck1;
     int64_t ck_stride;
     int64_t T;
-    int32_t ck_last;      // 1: the last chunk's end is kept too
-    int32_t S;            // steps of a chunk
-    int32_t H;            // halo of a window (>= S)
+    int32_t ck_steps;     // steps between two kept states (a divisor of S),
+    int32_t ck_split;     // > 0: and another state so many steps after each
+    int32_t S;            // steps of a chunk (<= the halo)
     int32_t nchunks;
     int32_t nwarps;
-    int32_t warp_values;  // shared-memory values of one warp
-    int32_t pad_;
     int32_t inject_warp, inject_chunk;  // test hook (-1: off)
-    int32_t cluster;      // 1: the grid is one thread-block cluster
-    ulonglong2* xbuf;     // exchange slots [CTA][side][parity][H * words]
-    unsigned long long epoch;  // of this launch, part of the slots' tags
-    DevError* err;
-    long long wait_ns;
+};
+
+template <typename Real>
+struct ResAdjProb {
+    int64_t base;      // the problem's first point in the kept span states
+    int64_t nx;
+    const Real* fA;
+    const Real* fB;
+    const Real* wbar;  // cotangent, T + 1 values
+    Real* grad;        // dL/dfA
+    Real c2, k;
+    int32_t js;        // receiver (-1: on a node, no adjoint)
+    int32_t pad_;
+};
+
+// The resident adjoint sweep (resident_adjoint.cu).
+template <typename Real>
+struct ResAdjParams {
+    ResExchange x;
+    const ResAdjProb<Real>* problems;
+    const ResWarp* warps;
+    const Real* uck0;   // forward state pair at the start of part x: uck + x ck_stride
+    const Real* uck1;
+    int64_t ck_stride;
+    int64_t T;
+    double* sums;       // [nwarps]: sum of lambda^{n+1}_j lap(u^n)_j over the warp's points
+    int32_t nspans, nwarps;
+    int32_t span;       // steps of a span
+    int32_t split;      // > 0: a span in two parts, the first of so many steps
+    int32_t parts;      // parts of the sweep (state x at the start of part x)
+    int32_t E;          // spans between two exchanges (halo >= E span)
 };
 
 struct VariantInfo {
@@ -275,6 +312,19 @@ cudaError_t res_occupancy(int dtype, int form, int P, int threads, size_t smem, 
 cudaError_t res_clusters(int dtype, int form, int P, int grid, int threads, size_t smem, int* clusters);
 cudaError_t res_launch(int dtype, int form, int P, const void* params, int grid, int threads, size_t smem,
                        bool cluster, cudaStream_t s);
+
+// any kernel over resident warps: one cooperative grid, or one cluster
+cudaError_t res_kernel_clusters(const void* fn, int grid, int threads, size_t smem, int* clusters);
+cudaError_t res_launch_kernel(const void* fn, const void* params, int grid, int threads, size_t smem, bool cluster,
+                              cudaStream_t s);
+
+// resident_adjoint.cu
+int radj_variants();
+void radj_info(int v, int* dtype, int* form, int* P, int* SA, int* max_warps);
+size_t radj_smem_bytes(int v, int H, int warps, int* warp_values);
+cudaError_t radj_fits(int v, size_t smem, bool* ok);
+cudaError_t radj_clusters(int v, int grid, int threads, size_t smem, int* clusters);
+cudaError_t radj_launch(int v, const void* params, int grid, int threads, size_t smem, bool cluster, cudaStream_t s);
 
 // adjoint_kernel.cu
 int adj_variant_count();
