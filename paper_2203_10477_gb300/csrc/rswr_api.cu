@@ -2286,6 +2286,52 @@ namespace {
 // span of an input boundary ("zones") are re-solved with the paper's rule
 // (rswr_resolve_kernel, from the span-start state into scratch, scattered into
 // the result).  Same bits as re-solving every window.
+//
+// FP32 runs whose windows fit a warp's registers take paper_run_kernel instead:
+// the same pieces, the whole run in one launch.
+
+// The pieces of paper_run_kernel: the kept points of subdomain i (from its left
+// neighbour's window end on) that an input boundary can reach in a span (of cap
+// steps at most) by the paper's rule, the grid's ends, and the rest.
+std::vector<PaperPiece> paper_pieces(const ProbHost& ph, int64_t cap, const PaperRunChoice& c,
+                                     int64_t* npair)
+{
+    const int64_t nx = ph.nx, N = ph.n_sub, el = (ph.ov + 1) / 2, er = ph.ov / 2;
+    std::vector<PaperPiece> v;
+    auto cut = [&](int64_t lo, int64_t hi, int64_t most, int32_t sub) {  // equal parts of at most `most`
+        if (hi <= lo) return;
+        const int64_t n = (hi - lo + most - 1) / most;
+        for (int64_t k = 0; k < n; ++k) {
+            const int64_t a = lo + (hi - lo) * k / n, b = lo + (hi - lo) * (k + 1) / n;
+            v.push_back(PaperPiece{a, (int32_t)(b - a), sub});
+        }
+    };
+    int64_t from = 0;
+    for (int64_t i = 0; i < N; ++i) {
+        const int64_t L = std::max<int64_t>(i * nx / N - el, 0);
+        const int64_t R = std::min<int64_t>((i + 1) * nx / N - 1 + er, nx - 1);
+        const int64_t z0 = i > 0 ? std::min(std::max(from, L + cap), R + 1) : from;  // [from, z0): left zone
+        const int64_t z1 = i + 1 < N ? std::max(z0, R + 1 - cap) : R + 1;            // [z1, R]: right zone
+        if (z1 > z0) {
+            cut(from, z0, c.edge, (int32_t)i);
+            const int64_t a = std::min(std::max(z0, cap), z1), b = std::max(a, std::min(z1, nx - cap));
+            cut(z0, a, c.edge, kPieceEnd);
+            cut(a, b, c.bulk, kPieceBulk);
+            cut(b, z1, c.edge, kPieceEnd);
+            cut(z1, R + 1, c.edge, (int32_t)i);
+        } else {
+            cut(from, R + 1, c.edge, (int32_t)i);
+        }
+        from = R + 1;
+    }
+    // short pieces first, two to a warp
+    const auto mid = std::stable_partition(v.begin(), v.end(), [&](const PaperPiece& x) {
+        return x.sub != kPieceBulk && x.len <= c.half;
+    });
+    *npair = (mid - v.begin()) / 2;
+    return v;
+}
+
 template <typename Real>
 rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, const Real* q0, const Real* q1, Real* out0,
                       Real* out1, int64_t* spans, int64_t spans_cap, int64_t* nspans, double beta, cudaStream_t s)
@@ -2323,9 +2369,15 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             }
     }
     const int64_t nt = (int64_t)tsub.size();
+    PaperRunChoice rc;
+    std::vector<PaperPiece> pieces;
+    int64_t npair = 0;
+    if (sizeof(Real) == 4 && T > 0 && e->inject_tile < 0 &&
+        paper_run_choose(e->form, nx, ov, cap, tau_max, e->num_sms, &rc))
+        pieces = paper_pieces(ph, cap, rc, &npair);
     // workspace: the zones' scratch pair, flux waveforms, tiles, span word
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
-    const size_t b_state = up(es * nx);
+    const size_t b_state = pieces.empty() ? up(es * nx) : 0;  // (paper_run_kernel needs no scratch pair)
     const size_t b_g = up(es * N * tau_max);
     const size_t b_t = up(sizeof(int64_t) * std::max<int64_t>(nt, 1));
     // the span kernel runs nsub spans of S steps per paper span (the last ones
@@ -2336,7 +2388,8 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
     const size_t b_samp = up(es * (size_t)nsamp);
     const int64_t rec_cap = spans ? std::min<int64_t>(spans_cap, std::max<int64_t>(T, 1)) : 0;
     const size_t b_rec = up(sizeof(int64_t) * (size_t)std::max<int64_t>(rec_cap, 1));
-    const size_t need = 2 * b_state + 2 * b_g + 3 * b_t + 256 + 2 * b_samp + b_rec + up(sizeof(PaperState));
+    const size_t b_one = 2 * b_state + 2 * b_g + 3 * b_t + 256 + 2 * b_samp + b_rec + up(sizeof(PaperState));
+    const size_t need = b_one + up(sizeof(PaperPiece) * pieces.size());
     if (need > e->adj_mem_cap) {
         RSWR_CUDA(cudaStreamSynchronize(s));
         cudaFree(e->adj_mem);
@@ -2359,7 +2412,7 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
     Real* d_fBs = reinterpret_cast<Real*>(m2 + b_samp);
     int64_t* d_rec = reinterpret_cast<int64_t*>(m2 + 2 * b_samp);
     PaperState* d_st = reinterpret_cast<PaperState*>(m2 + 2 * b_samp + b_rec);
-    if (nt > 0) {
+    if (nt > 0 && pieces.empty()) {
         RSWR_CUDA(cudaMemcpyAsync(d_sub, tsub.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, s));
         RSWR_CUDA(cudaMemcpyAsync(d_lo, tlo.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, s));
         RSWR_CUDA(cudaMemcpyAsync(d_hi, thi.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, s));
@@ -2420,6 +2473,49 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
         h0.done = T <= 0 ? 1 : 0;
         *e->h_pstate = h0;
         RSWR_CUDA(cudaMemcpyAsync(d_st, e->h_pstate, sizeof(PaperState), cudaMemcpyHostToDevice, s));
+    }
+    if constexpr (sizeof(Real) == 4) {
+        if (!pieces.empty()) {
+            PaperRun q{};
+            PaperPiece* const d_pieces = reinterpret_cast<PaperPiece*>(m + b_one);
+            q.pieces = d_pieces;
+            q.npiece = (int64_t)pieces.size();
+            q.npair = npair;
+            q.st = d_st;
+            q.arrived = reinterpret_cast<unsigned*>(d_span + 2);
+            q.err = e->d_err;
+            q.spans = rec_cap > 0 ? d_rec : nullptr;
+            q.spans_cap = rec_cap;
+            q.wait_ns = (long long)(e->wait_s * 1e9);
+            q.T = T;
+            q.beta_m = beta_m;
+            q.swap_u = static_cast<Real*>(e->q0[1]) - static_cast<Real*>(e->q0[0]);
+            q.swap_w = static_cast<Real*>(e->q1[1]) - static_cast<Real*>(e->q1[0]);
+            q.cap = (int32_t)cap;
+            q.steps = (int32_t)std::min<int64_t>(tau, T);
+            q.warp_values = rc.warp_values;
+            pp.u = static_cast<Real*>(e->q0[0]) + ph.base;
+            pp.w = static_cast<Real*>(e->q1[0]) + ph.base;
+            pp.uo = out0;
+            pp.wo = out1;
+            // both span words (bytes 0x7f: a value above any span), the grid barrier
+            RSWR_CUDA(cudaMemsetAsync(d_span, 0x7f, 2 * sizeof(int), s));
+            RSWR_CUDA(cudaMemsetAsync(d_span + 2, 0, sizeof(int), s));
+            RSWR_CUDA(cudaMemcpyAsync(d_pieces, pieces.data(), sizeof(PaperPiece) * pieces.size(),
+                                      cudaMemcpyHostToDevice, s));
+            if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
+            RSWR_CUDA(paper_run_launch(rc, pp, q, e->num_sms, s));
+            if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+            RSWR_CUDA(cudaMemcpyAsync(e->h_pstate, d_st, sizeof(PaperState), cudaMemcpyDeviceToHost, s));
+            rswr_status st = check_engine(e, s, nullptr, nullptr, nullptr);
+            if (st != RSWR_OK) return st;
+            const int64_t taken = e->h_pstate->count;
+            if (spans && taken > 0)
+                RSWR_CUDA(cudaMemcpy(spans, d_rec, sizeof(int64_t) * (size_t)std::min<int64_t>(taken, rec_cap),
+                                     cudaMemcpyDeviceToHost));
+            if (nspans) *nspans = taken;
+            return RSWR_OK;
+        }
     }
     pp.st = d_st;
     pp.steps = (int32_t)tau_max;  // (sizes only: the kernels take steps and span from d_st)

@@ -186,6 +186,34 @@ struct PaperParams {
     const PaperState* st;  // non-null: n0, steps and the span come from here (n0 / steps above unused)
 };
 
+// A piece of the grid that one warp updates per span: points [lo, lo + len) of
+// subdomain `sub` by the paper's rule, or by the bare stencil.
+struct PaperPiece {
+    int64_t lo;
+    int32_t len, sub;
+};
+constexpr int32_t kPieceBulk = -2, kPieceEnd = -1;  // (an end of the grid: nodes, no input boundary)
+
+// What paper_run_kernel needs beside PaperParams (span_min: two words there,
+// u / w the first state buffer, uo / wo the caller's arrays).
+struct PaperRun {
+    const PaperPiece* pieces;
+    PaperState* st;
+    unsigned* arrived;  // grid barrier (0 at launch)
+    DevError* err;
+    int64_t* spans;     // selected spans (null: not recorded)
+    long long wait_ns;
+    int64_t spans_cap, npiece, npair;  // pieces: npair pairs, then single ones
+    int64_t T, beta_m, swap_u, swap_w;  // swap: from the first to the second state buffer
+    int32_t cap, steps, warp_values;
+};
+
+struct PaperRunChoice {
+    int v = -1;
+    int64_t edge = 0, half = 0, bulk = 0;  // points of a piece at most (half: of one of a pair)
+    int warp_values = 0;
+};
+
 // ---- resident warp windows (resident.cuh) -------------------------------------
 
 constexpr int kResMaxHalo = 64;     // steps between two exchanges at most
@@ -358,6 +386,9 @@ cudaError_t paper_select_launch(int dtype, PaperState* st, const int* word, int 
                                 void* fAs, void* fBs, int nsamp, int64_t T, int64_t* spans, int64_t spans_cap,
                                 cudaStream_t s);
 cudaError_t paper_advance_launch(PaperState* st, int64_t T, int64_t beta_m, int64_t tau_max, cudaStream_t s);
+bool paper_run_choose(int form, int64_t nx, int64_t ov, int64_t cap, int64_t tau_max, int num_sms, PaperRunChoice* out);
+cudaError_t paper_run_launch(const PaperRunChoice& c, const PaperParams<float>& p, const PaperRun& q, int num_sms,
+                             cudaStream_t s);
 cudaError_t paper_resolve_launch(int dtype, const void* params, int ntiles, size_t smem, cudaStream_t s);
 
 // rswr_api.cu: sets the message returned by rswr_last_error_message()
