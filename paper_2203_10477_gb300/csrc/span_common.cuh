@@ -539,73 +539,115 @@ __device__ __forceinline__ void warp_neighbours(const Real (&u)[P], Real& lft, R
     if (lane == 31) rgt = u[P - 2];
 }
 
-// `steps` leapfrog steps of a warp window (neighbours by shuffles, mirror
-// ghosts at the window's ends) in the order: the thread's two end points, the
-// shuffles of their new values for the next step, then the interior points,
-// so that the shuffle latency hides behind the interior updates.  Every update
-// is the same expression on the same operands as leap_step(), so the bits are
-// identical.  `rec(u, lft, rgt, s)` sees every level s = 0 .. steps-1 with its
-// neighbours before it is advanced (probe recording; it must not shuffle).
+// A row of a probe buffer (shared address a): l at [3], the lane's points from
+// [4] on, r after them; stored without a branch (one that a single lane takes
+// costs a reconvergence each step).
+template <int P>
+__device__ __forceinline__ void st_row(bool on, uint32_t a, float l, const float (&u)[P], float r)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.f32 [%1 + 12], %2;\n\t@p st.shared.f32 [%3], %4;\n\t}" ::"r"((uint32_t)on),
+        "r"(a), "f"(l), "r"(a + (uint32_t)((P + 4) * sizeof(float))), "f"(r)
+        : "memory");
+    static_assert(P % 4 == 0, "whole vectors");
+#pragma unroll
+    for (int i = 0; i + 8 <= P; i += 8)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t"
+            "@p st.shared.v4.f32 [%1 + 16], {%6, %7, %8, %9};\n\t}" ::"r"((uint32_t)on),
+            "r"(a + (uint32_t)((i + 4) * sizeof(float))), "f"(u[i]), "f"(u[i + 1]), "f"(u[i + 2]), "f"(u[i + 3]),
+            "f"(u[i + 4]), "f"(u[i + 5]), "f"(u[i + 6]), "f"(u[i + 7])
+            : "memory");
+    if constexpr (P % 8 != 0)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(
+                         (uint32_t)on),
+                     "r"(a + (uint32_t)(P * sizeof(float))), "f"(u[P - 4]), "f"(u[P - 3]), "f"(u[P - 2]), "f"(u[P - 1])
+                     : "memory");
+}
+
+// What a free warp window holds besides plain points.
+enum : int {
+    kWinPlain = 0,
+    kWinNode = 1,    // a Dirichlet node
+    kWinSource = 2,  // a point source
+};
+
+// The samples of a warp's special point over a span of at most 32 steps: lane l
+// has the one of step l (level n0 + 1 + l); old: level n0 (a node's value).
+template <typename Real>
+struct WarpSamples {
+    Real c, old;
+    int r;  // the special point's register, -1: not on this lane
+};
+
 struct NoRecord {
     template <typename U, typename Real>
     __device__ __forceinline__ void operator()(const U&, Real, Real, int) const {}
 };
 
-template <typename Real, int FORM, int P, typename Rec = NoRecord>
+// `steps` leapfrog steps of a warp window (neighbours by shuffles; what enters
+// at its ends travels one point per step and stays inside the halo) in the order:
+// the thread's two end points, the shuffles of their new values for the next
+// step, then the interior points, so that the shuffle latency hides behind the
+// interior updates.  Every update is the same expression on the same operands as
+// leap_step() and patch_special(), so the bits are identical.  A special
+// point costs two or three predicated instructions per register and step.
+// `rec(u, lft, rgt, s)` sees every level s = 0 .. steps-1 with its neighbours
+// before it is advanced (probe recording; it must not shuffle).
+template <typename Real, int FORM, int P, int SPEC = kWinPlain, typename Rec = NoRecord>
 __device__ __forceinline__ void warp_steps_edges_first(Real (&u)[P], Real (&w)[P], Real c2, Real k, int steps,
-                                                       int lane, Rec rec = Rec{})
+                                                       Rec rec = Rec{},
+                                                       WarpSamples<Real> sp = WarpSamples<Real>{})
 {
     static_assert(P >= 3, "edges-first order needs interior points");
-    Real lft, rgt;
-    warp_neighbours<Real, P>(u, lft, rgt, lane);
+    Real lft = __shfl_up_sync(kFull, u[P - 1], 1);
+    Real rgt = __shfl_down_sync(kFull, u[0], 1);
     for (int s = 0; s < steps; ++s) {
         rec(u, lft, rgt, s);
-        Real n0, nl, v0, vl;  // new first / last point and their second components
-        Real d0 = Real(0);
-        if constexpr (FORM == kIncrement) {
-            d0 = rsub(u[1], u[0]);
-            const Real dm = rsub(u[P - 1], u[P - 2]);
-            v0 = rfma(c2, rsub(d0, rsub(u[0], lft)), w[0]);
-            vl = rfma(c2, rsub(rsub(rgt, u[P - 1]), dm), w[P - 1]);
-            n0 = radd(u[0], v0);
-            nl = radd(u[P - 1], vl);
-        } else {
-            n0 = rfma(c2, radd(lft, u[1]), rfma(k, u[0], -w[0]));
-            v0 = u[0];
-            nl = rfma(c2, radd(u[P - 2], rgt), rfma(k, u[P - 1], -w[P - 1]));
-            vl = u[P - 1];
+        Real x = Real(0), dx = Real(0);
+        if constexpr (SPEC != kWinPlain) x = __shfl_sync(kFull, sp.c, s & 31);
+        if constexpr (SPEC == kWinNode) {
+            dx = rsub(x, sp.old);
+            sp.old = x;
         }
-        Real nlft = __shfl_up_sync(kFull, nl, 1);
-        Real nrgt = __shfl_down_sync(kFull, n0, 1);
-        if constexpr (FORM == kIncrement) {
-            Real dprev = d0;
-#pragma unroll
-            for (int i = 1; i < P - 1; ++i) {
-                const Real d = rsub(u[i + 1], u[i]);
-                const Real v = rfma(c2, rsub(d, dprev), w[i]);
-                dprev = d;
-                w[i] = v;
-                u[i] = radd(u[i], v);
+        // point i from its neighbours and (increment form) the two differences
+        auto update = [&](int i, Real ul, Real ur, Real d, Real dprev, Real& un, Real& wn) {
+            const Real uc = u[i];
+            if constexpr (FORM == kIncrement) {
+                Real v = rfma(c2, rsub(d, dprev), w[i]);
+                if constexpr (SPEC == kWinSource) v = sp.r == i ? radd(v, x) : v;
+                un = radd(uc, v);
+                wn = v;
+                if constexpr (SPEC == kWinNode) {
+                    un = sp.r == i ? x : un;
+                    wn = sp.r == i ? dx : wn;
+                }
+            } else {
+                un = rfma(c2, radd(ul, ur), rfma(k, uc, -w[i]));
+                wn = uc;
+                if constexpr (SPEC == kWinSource) un = sp.r == i ? radd(un, x) : un;
+                if constexpr (SPEC == kWinNode) un = sp.r == i ? x : un;
             }
-        } else {
-            Real ul = u[0];
+        };
+        Real n0, nl, v0, vl;  // new first / last point and their second components
+        const Real d0 = rsub(u[1], u[0]), dm = rsub(u[P - 1], u[P - 2]);
+        update(0, lft, u[1], d0, rsub(u[0], lft), n0, v0);
+        update(P - 1, u[P - 2], rgt, rsub(rgt, u[P - 1]), dm, nl, vl);
+        lft = __shfl_up_sync(kFull, nl, 1);
+        rgt = __shfl_down_sync(kFull, n0, 1);
+        Real dprev = d0, ul = u[0];
 #pragma unroll
-            for (int i = 1; i < P - 1; ++i) {
-                const Real uc = u[i];
-                const Real un = rfma(c2, radd(ul, u[i + 1]), rfma(k, uc, -w[i]));
-                w[i] = uc;
-                u[i] = un;
-                ul = uc;
-            }
+        for (int i = 1; i < P - 1; ++i) {
+            const Real uc = u[i], ur = u[i + 1];
+            const Real d = rsub(ur, uc);
+            update(i, ul, ur, d, dprev, u[i], w[i]);
+            dprev = d;
+            ul = uc;
         }
         u[0] = n0;
         w[0] = v0;
         u[P - 1] = nl;
         w[P - 1] = vl;
-        if (lane == 0) nlft = u[1];
-        if (lane == 31) nrgt = u[P - 2];
-        lft = nlft;
-        rgt = nrgt;
     }
 }
 
@@ -613,8 +655,23 @@ __device__ __forceinline__ void warp_steps_edges_first(Real (&u)[P], Real (&w)[P
 template <typename Real, int P, int KH>
 __device__ __forceinline__ void owned_to_smem(Real* s, const Real (&r)[P], int own_lo, int own_hi)
 {
+    constexpr int N = Vec<Real, P>::N;
     if (KH == 0 || (own_lo == 0 && own_hi == P)) {
         regs_to_smem<Real, P>(s, r);
+    } else if constexpr (KH % N == 0) {
+        // (P and KH are whole vectors, so are a thread's owned points)
+#pragma unroll
+        for (int i = 0; i < P; i += N)
+            if (i >= own_lo && i < own_hi) {
+                typename Vec<Real, P>::T v;
+                v.x = r[i];
+                v.y = r[i + 1];
+                if constexpr (N == 4) {
+                    v.z = r[i + 2];
+                    v.w = r[i + 3];
+                }
+                *reinterpret_cast<typename Vec<Real, P>::T*>(s + i) = v;
+            }
     } else {
 #pragma unroll
         for (int i = 0; i < P; ++i)

@@ -185,12 +185,15 @@ struct Geom {
 // the window take it together.  The step loop is instantiated six times
 // (probes yes/no x {plain, special points, special points + user sources}) so
 // that a plain interior tile runs the bare stencil with no per-step tests.
-template <typename Real, int FORM, int P, int NW, int KH, int BAR, bool USRC>
+// Free warp windows (KH >= the span) take their own paths: see there.  They
+// record probes in free_u / free_w, this warp's owned points of the stage in
+// shared memory, once wait_free() says that every warp has read its window.
+template <typename Real, int FORM, int P, int NW, int KH, int BAR, bool USRC, typename Wait>
 __device__ __forceinline__ void predict_tile(const SpanParams<Real>& prm, const ProblemDev<Real>& pr,
                                              const TileDev& td, Real (&u)[P], Real (&w)[P], int64_t gj0, int64_t n0,
                                              int steps, int tb, int own_lo, int own_hi,
                                              const ProbeDev<Real>* tprobes, int np, Real* xch, Real* hx, int warp,
-                                             int lane, bool edge)
+                                             int lane, bool edge, Real* free_u, Real* free_w, Wait&& wait_free)
 {
     constexpr int CW = KH == 0 ? 32 * P : 32 * P - 2 * KH;
     constexpr int W = KH == 0 ? NW * 32 * P : NW * CW + 2 * KH;
@@ -299,18 +302,18 @@ __device__ __forceinline__ void predict_tile(const SpanParams<Real>& prm, const 
         if constexpr (KH > 0 && !SP) {
             if constexpr (!PR) {
                 // plain interior tile of a warp window: the bare stencil, edges first
-                warp_steps_edges_first<Real, FORM, P>(u, w, c2, kk, s_end - s_begin, lane);
+                warp_steps_edges_first<Real, FORM, P>(u, w, c2, kk, s_end - s_begin);
                 return;
             } else {
                 // interior tile with probes: edges first as well, each level
                 // recorded by its owner before it is advanced; a warp that owns
                 // none of the tile's probes runs the bare stencil (warp-uniform)
                 if (!many_probes && !__any_sync(kFull, nown > 0)) {
-                    warp_steps_edges_first<Real, FORM, P>(u, w, c2, kk, s_end - s_begin, lane);
+                    warp_steps_edges_first<Real, FORM, P>(u, w, c2, kk, s_end - s_begin);
                     return;
                 }
                 if (!many_probes) {
-                    warp_steps_edges_first<Real, FORM, P>(u, w, c2, kk, s_end - s_begin, lane, recf);
+                    warp_steps_edges_first<Real, FORM, P>(u, w, c2, kk, s_end - s_begin, recf);
                     return;
                 }
             }
@@ -399,7 +402,117 @@ __device__ __forceinline__ void predict_tile(const SpanParams<Real>& prm, const 
         }
     };
 
-    if constexpr (KH > 0) {
+    if constexpr (KH > 0 && P < 2 * KH) {
+        // Free warp windows: the warp halo covers the whole span (steps <= KH <=
+        // 32, checked by the caller), so warps never exchange data inside a span
+        // and each takes the loop that its own points need: a tile with a node,
+        // a source or probes keeps three bare warps and one that pays a few
+        // instructions per register.  Windows with two special points, and
+        // more than four probes, take the general loop.  A special tile used to run
+        // the general loop on all warps, some 0.8 us a step, and paced its
+        // neighbours: 4,194,304 points with ten sources, 1000 steps, 1327 -> 844 us;
+        // 2^24 points with all interface waveforms, 1280 steps, 3944 -> 3630 us.
+        static_assert(KH <= 32, "a lane holds a step's sample");
+        const int64_t wlo = gj - (int64_t)lane * P, wend = wlo + 32 * P;
+        const bool node_l = wlo <= 0 && wend > 0, node_r = wlo <= nx - 1 && wend > nx - 1;
+        int special = (int)node_l + (int)node_r;
+        int64_t sj = -1, sstride = 1;
+        const Real* sptr = nullptr;
+        if (has_src && pr.js >= wlo && pr.js < wend) {
+            ++special;
+            sj = pr.js;
+            sptr = pr.src;
+            sstride = pr.src_stride;
+        }
+        if constexpr (USRC)
+            for (int q = td.src_begin; q < td.src_end; ++q) {
+                const SrcDev<Real> sd = prm.srcs[q];
+                if (sd.j >= wlo && sd.j < wend) {
+                    ++special;
+                    sj = sd.j;
+                    sptr = sd.samples;
+                }
+            }
+        // probes: lanes 8 e .. 8 e + 7 turn the recorded levels of probe e into stores
+        constexpr int ROW = P + 8, LV = 8;  // a lane's points and neighbours; levels of a row buffer
+        static_assert(4 * LV * ROW <= 2 * (32 * P - 2 * KH), "row buffers fit the owned points");
+        int nrec = 0, slots = 0, lane_of[4] = {-1, -1, -1, -1};
+        int my_q = -1, my_slot = 0, my_r = 0;
+        for (int q = 0; q < (many_probes ? 0 : np); ++q) {
+            const int pos = (int)(tprobes[q].gidx - wabs) - warp * CW;
+            if (pos < (warp > 0 ? KH : 0) || pos >= (warp < NW - 1 ? 32 * P - KH : 32 * P)) continue;
+            const int ol = pos / P;
+            int sl = 0;
+            while (sl < slots && sl < 4 && lane_of[sl] != ol) ++sl;
+            if (sl == slots) {
+                if (sl < 4) lane_of[sl] = ol;
+                ++slots;
+            }
+            if (nrec == (lane >> 3)) {
+                my_q = q;
+                my_slot = sl;
+                my_r = pos - ol * P;
+            }
+            ++nrec;
+        }
+        if (special > 1 || many_probes || nrec > 4) {
+            run(Yes{}, Yes{}, std::bool_constant<USRC>{}, 0, steps);
+            return;
+        }
+        WarpSamples<Real> sp{Real(0), Real(0), -1};
+        if (special) {
+            const int64_t j = node_l ? 0 : (node_r ? nx - 1 : sj);
+            const Real* a = node_l ? pr.fA : (node_r ? pr.fB : sptr);
+            const int64_t st = node_l || node_r ? 1 : sstride;
+            if (j >= gj && j < gj + P) sp.r = (int)(j - gj);
+            sp.c = level_sample(a, st, n0 + 1 + lane, prm.T);
+            if (node_l || node_r) sp.old = level_sample(a, st, n0, prm.T);
+        }
+        auto slot_row = [&](int sl, int lv) { return (sl < 2 ? free_u : free_w) + ((sl & 1) * LV + lv) * ROW; };
+        auto steps_of = [&](auto spec, auto rec) {
+            warp_steps_edges_first<Real, FORM, P, decltype(spec)::value>(u, w, c2, kk, steps, rec, sp);
+        };
+        auto all_steps = [&](auto rec) {
+            if (special == 0) steps_of(std::integral_constant<int, kWinPlain>{}, rec);
+            else if (node_l || node_r) steps_of(std::integral_constant<int, kWinNode>{}, rec);
+            else steps_of(std::integral_constant<int, kWinSource>{}, rec);
+        };
+        if (nrec == 0) {
+            all_steps(NoRecord{});
+        } else {
+            wait_free();
+            Real* row = nullptr;
+#pragma unroll
+            for (int sl = 0; sl < 4; ++sl)
+                if (lane_of[sl] == lane) row = slot_row(sl, 0);
+            const uint32_t row0 = row ? smem_addr(row) : smem_addr(free_u);
+            const bool on = row != nullptr;
+            OwnedProbe<Real> op{};
+            if (my_q >= 0) op = own_probe<Real>(tprobes[my_q], wabs, tb, n0, steps);
+            const Real* const my_row = slot_row(my_slot, lane & 7);
+            auto flush = [&](int first) {  // levels first .. first + 7 of the span
+                __syncwarp();
+                const int s = first + (lane & 7);
+                if (my_q >= 0 && s < op.count) {
+                    const Real um = my_row[3 + my_r], uc = my_row[4 + my_r], up = my_row[5 + my_r];
+                    const Real val = op.kind == 0 ? uc : rsub(up, um);
+                    op.ptr[s * op.stride] = rmul(val, op.scale);
+                }
+                __syncwarp();
+            };
+            all_steps([&](const Real(&uu)[P], Real l, Real r, int s) {
+                if ((s & (LV - 1)) == 0 && s > 0) flush(s - LV);
+                st_row<P>(on, row0 + (uint32_t)((s & (LV - 1)) * ROW * sizeof(Real)), l, uu, r);
+            });
+            if (steps > 0) flush((steps - 1) & ~(LV - 1));
+        }
+        if (node_r) {  // points outside the grid stay 0 (see make_special)
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+                if (gj + i > nx - 1) u[i] = w[i] = Real(0);
+        }
+        return;
+    } else if constexpr (KH > 0) {
         if constexpr (P >= 2 * KH) {
             // warp halos refreshed every KH steps
             for (int s0 = 0; s0 < steps; s0 += KH) {
@@ -409,10 +522,6 @@ __device__ __forceinline__ void predict_tile(const SpanParams<Real>& prm, const 
                 }
                 run_steps(s0, (s0 + KH < steps) ? s0 + KH : steps);
             }
-        } else {
-            // free warp windows: the warp halo covers the whole span (steps <= KH,
-            // checked by the caller), so warps never exchange data inside a span
-            run_steps(0, steps);
         }
     } else {
         if (!slow && !has_usrc && !has_probe) {
@@ -550,7 +659,7 @@ __global__ void __launch_bounds__(NT, MINB) span_kernel(const __grid_constant__ 
         }
 
         predict_tile<Real, FORM, P, NW, KH, 0, USRC>(prm, pr, td, u, w, gj0, n0, steps, tb, own_lo, own_hi, s_probes,
-                                                  np, xch, hx, warp, lane, edge);
+                                                  np, xch, hx, warp, lane, edge, nullptr, nullptr, [] {});
 
         // ---- select + update: write the window back, store only the core
         __syncthreads();  // every thread has read its window (KH > 0: windows overlap)
@@ -863,18 +972,22 @@ __global__ void __launch_bounds__(NT + 32, MINB) span_kernel_ws(const __grid_con
         if (si.ticket < 0) break;
 
         const int steps = si.steps;
+        // every warp has read its window from stage y
+        auto wait_read = [&]() {
+            if (!mbar_wait_bounded(&read_bar[y], (rpar >> y) & 1u, prm.wait_ns, &prm.err->code))
+                latch_error(prm.err, kDevTimeoutLoad, si.tile, si.k, 0);
+        };
         if (kFree && steps > KH) {
             // the host never schedules a span longer than a free variant's warp halo
             if (tid == 0) latch_error(prm.err, kDevBadTicket, si.tile, si.k, 0);
         } else {
             predict_tile<Real, FORM, P, NW, KH, NT, USRC>(prm, si.pr, si.td, u, w, si.gj0, si.n0, steps, tb, own_lo,
                                                        own_hi, s_probes[y], si.np, xch, hx, warp, lane,
-                                                       si.edge != 0);
+                                                       si.edge != 0, su + warp * G::CW + KH, sw + warp * G::CW + KH,
+                                                       wait_read);
         }
         if constexpr (kFree) {
-            // every warp has read its window from stage y before anyone overwrites it
-            const bool rd = mbar_wait_bounded(&read_bar[y], (rpar >> y) & 1u, prm.wait_ns, &prm.err->code);
-            if (!rd) latch_error(prm.err, kDevTimeoutLoad, si.tile, si.k, 0);
+            wait_read();  // ... before anyone overwrites it
         }
         rpar ^= 1u << y;
         owned_to_smem<Real, P, KH>(su + tb, u, own_lo, own_hi);
