@@ -1210,7 +1210,8 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
 }
 
 // Whether a run takes the resident path, and its cut.  A plan whose variant is
-// a resident one always does (or the run is refused); a plan as it was created
+// a resident one does, or takes the default variant where the grid is a little too
+// large (far too large: the run is refused); a plan as it was created
 // does when its grid fits on the chip; a variant, span or mode chosen by the
 // caller or the autotuner is kept to.
 rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
@@ -1220,9 +1221,11 @@ rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
     const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
     if (r.mono || r.from_state || r.steps_dev || r.T <= 0 || r.T >= ((int64_t)1 << 31) - 256) return RSWR_OK;
     if (vi.resident) {
-        if (!res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp))
+        *take = res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp);
+        // (grids that a wider tiling of these variants once held still run, with tickets)
+        const int64_t most = (int64_t)e->num_sms * (e->dtype == kF32 ? 13312 : 3968);
+        if (!*take && (e->packed_len > most || e->inject_tile >= 0))
             return fail(RSWR_ENOTSUP, "resident variant: the grid does not fit on the GPU at once");
-        *take = true;
     } else if (!e->chosen && e->mode == RSWR_MODE_PERSISTENT && e->inject_tile < 0) {
         *take = res_choose(e, 0, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp);
     }
@@ -2199,12 +2202,27 @@ rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cu
 {
     if (probe_steps < 1) return fail(RSWR_EINVAL, "probe_steps must be >= 1");
     const int S_max = span_limit(e);
-    const std::string key = tune_key(e, S_max);
+    std::string key = tune_key(e, S_max);
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         tune_load();
         auto it = g_tune.find(key);
-        if (use_cache && it != g_tune.end()) {
+        // an entry that names no variant of this dtype and form is no choice; a
+        // resident choice of a smaller grid of the class may not fit this one
+        auto usable = [&](const TuneChoice& c) {
+            if (c.variant < 0 || c.variant >= span_variant_count()) return false;
+            const VariantInfo vi = span_variant_info(c.variant);
+            return vi.dtype == e->dtype && vi.form == e->form;
+        };
+        ResPlan rp;
+        if (it != g_tune.end() && usable(it->second)) {
+            const VariantInfo vi = span_variant_info(it->second.variant);
+            if (vi.resident && !res_choose(e, vi.P, it->second.S, kResMaxHalo, false, false, false, &rp)) {
+                key += ":x";
+                it = g_tune.find(key);
+            }
+        }
+        if (use_cache && it != g_tune.end() && usable(it->second)) {
             rswr_status st = apply_choice(e, it->second);
             if (st == RSWR_OK) {
                 if (variant) *variant = e->variant;
@@ -2233,12 +2251,14 @@ rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cu
     r.T = probe_steps;
     r.out0 = e->d_scratch[0];
     r.out1 = e->d_scratch[1];
+    ResPlan fit;
     std::vector<int> spans{S_max};
     if (S_max / 2 >= 4) spans.push_back(S_max / 2);
     for (int v = 0; v < span_variant_count(); ++v) {
         const VariantInfo vi = span_variant_info(v);
         if (vi.dtype != e->dtype || vi.form != e->form) continue;
         for (int S : spans) {
+            if (vi.resident && !res_choose(e, vi.P, S, kResMaxHalo, false, false, false, &fit)) continue;
             for (int mode = 0; mode < (vi.resident ? 1 : 2); ++mode) {  // (one mode for resident windows)
                 if (apply_choice(e, TuneChoice{v, mode, S}) != RSWR_OK) continue;
                 if (run_engine(e, r, s) != RSWR_OK) continue;  // warm-up (and graph capture)

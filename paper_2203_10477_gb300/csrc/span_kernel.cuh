@@ -1029,11 +1029,11 @@ __global__ void __launch_bounds__(NT + 32, MINB) span_kernel_ws(const __grid_con
     X(PLAIN, double, kCanonical, 8, 128, 0, 4)         \
     X(PLAIN, double, kCanonical, 8, 256, 0, 2)         \
     X(PLAIN, double, kIncrement, 8, 256, 0, 2)         \
-    X(RES, float, kIncrement, 8, 128, 0, 1)            \
-    X(RES, float, kIncrement, 16, 128, 0, 1)           \
     X(RES, float, kIncrement, 32, 128, 0, 1)           \
-    X(RES, float, kIncrement, 4, 128, 0, 1)            \
+    X(RES, float, kIncrement, 16, 128, 0, 1)           \
     X(RES, double, kCanonical, 8, 128, 0, 1)           \
+    X(RES, float, kIncrement, 8, 128, 0, 1)            \
+    X(RES, float, kIncrement, 4, 128, 0, 1)            \
     X(RES, double, kCanonical, 16, 128, 0, 1)          \
     X(RES, double, kCanonical, 12, 128, 0, 1)          \
     X(RES, double, kCanonical, 4, 128, 0, 1)           \

@@ -106,3 +106,23 @@ def test_sources_in_resident_windows(R, oracle_mod, dtype, places):
     same(host(out["u"]), ref["u"], "u")
     same(host(out["w"]), ref["w"], "w")
     same(host(out["recv"]), ref["rec"][0], "receiver")
+
+
+def test_grids_just_above_the_capacity_still_run(R, oracle_mod):
+    """A resident variant chosen by the caller, or remembered from a smaller grid of
+    the same size class by the autotuner, on a grid that does not fit at once."""
+    nx, T = 1400003, 40
+    dt, fA, fB, q0, q1, kw = problem(oracle_mod, F32, nx, T)
+    ref = oracle_mod.leapfrog(nx, T, 1.0, dt, fA, fB, q0=q0, q1=q1, **kw)
+    R.Plan(0.0, 1.0, 1.0, 1 << 20, dt, 64, 60, dtype=F32).autotune(64)
+    for v in [None] + [v["variant"] for v in R.variants() if v["dtype"] == F32 and v["resident"]]:
+        plan = R.Plan(0.0, 1.0, 1.0, nx, dt, 64, 60, dtype=F32)
+        plan.set_span(30)
+        if v is None:
+            plan.autotune(64)
+        else:
+            plan.set_variant(v)
+        out = plan.run(fA, fB, T, q0=q0, q1=q1)
+        plan.check()
+        same(host(out["u"]), ref["u"], f"variant {v} u")
+        same(host(out["w"]), ref["w"], f"variant {v} w")
