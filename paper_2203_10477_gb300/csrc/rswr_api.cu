@@ -100,6 +100,8 @@ struct Engine {
     int64_t ck_spacing = 0;  // adjoint checkpoint spacing in spans (0: automatic)
     int S = 1, H = 4, W = 0, core = 0, P = 0, NT = 0;
     int inject_tile = -1, inject_span = -1;
+    int pass = 1;           // steps of a launch's span: whole spans of S (layout)
+    bool span_set = false;  // the caller chose S
     bool is_plan = true;
     bool part = false;  // a part [lo, hi) of a larger grid (rswr_plan_create_part)
 
@@ -228,7 +230,16 @@ rswr_status layout(Engine* e)
     e->P = vi.P;
     e->NT = vi.NT;
     e->W = vi.W;
-    e->H = (e->S + 3) / 4 * 4;
+    // FP32 spans of 16 steps and fewer (overlaps below 64) are bound by the state's
+    // way to memory and back: a pass of the span kernel takes as many whole spans
+    // as 32 steps hold (its windows' own halos are as wide as the pass), unless the
+    // caller chose the span.  512 uneven problems of overlap 32: 8382 -> 6871 us;
+    // FP64 is bound by its pipe.
+    int m = 1;
+    if (e->dtype == kF32 && !vi.resident && !e->span_set && e->inject_tile < 0)
+        for (m = std::max(1, 32 / e->S); m > 1 && !variant_takes_span(vi, e->S * m);) --m;
+    e->pass = e->S * m;
+    e->H = (e->pass + 3) / 4 * 4;
     e->core = e->W - 2 * e->H;
     if (!variant_takes_span(vi, e->S)) return fail(RSWR_EINVAL, "span longer than the warp halo of this variant");
     if (e->core < e->H || e->core < 4) return fail(RSWR_EINVAL, "span too long for the CTA window of this variant");
@@ -633,7 +644,7 @@ SpanParams<Real> span_params(Engine* e, int64_t T, int nspans)
     prm.T = T;
     prm.H = e->H;
     prm.core = e->core;
-    prm.S = e->S;
+    prm.S = e->pass;
     prm.nspans = nspans;
     prm.span = -1;
     prm.inject_tile = e->inject_tile;
@@ -691,7 +702,7 @@ rswr_status device_work(Engine* e, const RunReq& r, int nprobe, int64_t mono_blk
     const void* fin1;
     if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
     if (!r.mono) {
-        const int nspans = (int)((r.T + e->S - 1) / e->S);
+        const int nspans = (int)((r.T + e->pass - 1) / e->pass);
         SpanParams<Real> prm = span_params<Real>(e, r.T, nspans);
         prm.steps_dev = r.steps_dev;
         int bps = 0;
@@ -2261,6 +2272,7 @@ rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cu
             if (vi.resident && !res_choose(e, vi.P, S, kResMaxHalo, false, false, false, &fit)) continue;
             for (int mode = 0; mode < (vi.resident ? 1 : 2); ++mode) {  // (one mode for resident windows)
                 if (apply_choice(e, TuneChoice{v, mode, S}) != RSWR_OK) continue;
+                if (S < S_max && e->pass >= S_max) continue;  // (the same passes as with S_max)
                 if (run_engine(e, r, s) != RSWR_OK) continue;  // warm-up (and graph capture)
                 RSWR_CUDA(cudaEventRecord(a, s));
                 rswr_status st = run_engine(e, r, s);
@@ -2403,8 +2415,8 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
     // the span kernel runs nsub spans of S steps per paper span (the last ones
     // may take fewer or none: the span is chosen on the device), reading the
     // span's boundary samples from a copy of nsamp levels
-    const int64_t nsub = (cap + e->S - 1) / e->S;
-    const int nsamp = (int)(nsub * e->S + 1);
+    const int64_t nsub = (cap + e->pass - 1) / e->pass;
+    const int nsamp = (int)(nsub * e->pass + 1);
     const size_t b_samp = up(es * (size_t)nsamp);
     const int64_t rec_cap = spans ? std::min<int64_t>(spans_cap, std::max<int64_t>(T, 1)) : 0;
     const size_t b_rec = up(sizeof(int64_t) * (size_t)std::max<int64_t>(rec_cap, 1));
@@ -2565,7 +2577,7 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             RunReq r;
             r.fA = fA ? d_fAs : nullptr;
             r.fB = fB ? d_fBs : nullptr;
-            r.T = nsub * e->S;
+            r.T = nsub * e->pass;
             r.steps_dev = &d_st->span;
             r.from_state = true;
             rswr_status st = run_impl<Real>(e, r, s);
@@ -2705,13 +2717,16 @@ rswr_status rswr_plan_set_span(rswr_plan_t plan, int32_t S)
     if (S < 1 || S > e->probs[0].ov / 2 || S > kSpanCap)
         return fail(RSWR_EOVERLAP, "span must satisfy 1 <= S <= floor(overlap/2)");
     const int old = e->S, oldv = e->variant;
+    const bool old_set = e->span_set;
     e->S = S;
+    e->span_set = true;
     // a variant whose warp halo is shorter than S gives way to the default one for S
     if (!variant_takes_span(span_variant_info(e->variant), S)) e->variant = default_variant(e->dtype, e->form, S);
     rswr_status st = e->variant >= 0 ? layout(e) : fail(RSWR_ENOTSUP, "no kernel variant runs this span");
     if (st != RSWR_OK) {
         e->S = old;
         e->variant = oldv;
+        e->span_set = old_set;
         layout(e);
     } else {
         e->chosen = true;
@@ -2759,9 +2774,19 @@ rswr_status rswr_plan_set_sources(rswr_plan_t plan, int64_t nsrc, const int64_t*
 rswr_status rswr_plan_inject_missing_flag(rswr_plan_t plan, int32_t tile, int32_t span)
 {
     if (!plan) return fail(RSWR_EINVAL, "NULL plan");
-    if (tile >= plan->e->ntiles) return fail(RSWR_EINVAL, "tile out of range");
-    plan->e->inject_tile = tile < 0 ? -1 : tile;
-    plan->e->inject_span = span;
+    Engine* e = plan->e;
+    const int old = e->inject_tile;
+    e->inject_tile = tile < 0 ? -1 : tile;
+    // (tiles and spans are those of the one-span tiling)
+    const bool retile = (old < 0) != (tile < 0) && e->dtype == kF32 && !e->span_set && e->S <= 16;
+    rswr_status st = retile ? layout(e) : RSWR_OK;
+    if (st == RSWR_OK && tile >= e->ntiles) st = fail(RSWR_EINVAL, "tile out of range");
+    if (st != RSWR_OK) {
+        e->inject_tile = old;
+        if (retile) layout(e);
+        return st;
+    }
+    e->inject_span = span;
     return RSWR_OK;
 }
 

@@ -64,3 +64,32 @@ def test_special_points_equal_oracle(R, oracle_mod, form, tail):
             for a, b in (("u", ref["u"]), ("w", ref["w"]), ("traces", ref["traces"]), ("recv", mono["rec"][0])):
                 bad = np.flatnonzero(got[a].cpu().numpy().ravel() != np.asarray(b).ravel())
                 assert bad.size == 0, (v, js, a, bad[:5])
+
+
+@pytest.mark.parametrize("ov", [4, 11, 16, 21, 32, 33, 63, 64])
+def test_passes_of_several_spans_equal_oracle(R, oracle_mod, ov):
+    """Overlaps below 64: a pass holds as many whole spans as 32 steps (ov // 2 steps
+    each) for plans whose span the caller did not choose; tuned, batched, with
+    a fault injected (one span to a pass again) and taken back."""
+    nx, N, T = 9001, 40, 150
+    dt = 0.9 / (nx - 1)
+    r = inputs.rng(ov)
+    fA, fB = (r.standard_normal(T + 1).astype(np.float32) for _ in range(2))
+    q0, q1 = (r.standard_normal(nx).astype(np.float32) for _ in range(2))
+    ref = oracle_mod.rswr_mask(nx, T, 1.0, dt, fA, fB, N, ov, q0=q0, q1=q1, form=1, prec="f32")
+    S = ov // 2
+    plan = R.Plan(0.0, 1.0, 1.0, nx, dt, N, ov, dtype=F32)
+    plan.set_mode(1)  # (not the resident path)
+    plan.set_variant(0)
+    halos = []
+    for step in range(3):
+        plan.inject_missing_flag(2 if step == 1 else -1, 1 << 30)  # (a span that the run does not reach)
+        halos.append(plan.info()["halo"])
+        assert plan.info()["span_steps"] == S
+        got = plan.run(fA, fB, T, q0=q0, q1=q1, traces=True)
+        plan.check()
+        for k in ("u", "w", "traces"):
+            assert np.array_equal(got[k].cpu().numpy(), ref[k]), (k, step)
+    assert halos == [(m + 3) // 4 * 4 for m in (32 // S * S, S, 32 // S * S)]
+    plan.set_span(S)
+    assert plan.info()["halo"] == (S + 3) // 4 * 4
