@@ -545,19 +545,25 @@ struct Exchange {
     // did).  mute: this warp publishes nothing (test hook).
     __device__ __forceinline__ bool swap(const ResExchange& x, Real (&u)[P], Real (&w)[P], int k, bool mute)
     {
-        // this warp's window to shared memory, and the H owned
-        // points next to an end that has its neighbour in another CTA onwards
+        // the H owned points next to each end to shared memory, and those next to
+        // an end that has its neighbour in another CTA onwards
         const int par = k & 1;
         const unsigned long long tag = (x.epoch << 32) | (unsigned)(k + 1);
         Real* const win = area + par * 64 * P;
-        if constexpr (P * sizeof(Real) % 16 == 0) {
-            span::regs_to_smem<Real, P>(win + lane * P, u);
-            span::regs_to_smem<Real, P>(win + 32 * P + lane * P, w);
-        } else {
+        // (with 64 bytes and more to a lane, from the few lanes that hold them only: 32
+        // lanes at that stride meet in the same banks; 1,048,576 FP32 points, 2048
+        // steps, 439 -> 402 us.  Below, the branch costs more than the conflicts.)
+        const int p0 = lane * P;
+        if (P * sizeof(Real) < 64 || (left && p0 < a0 + H && p0 + P > a0) || (right && p0 < a0 + len && p0 + P > a0 + len - H)) {
+            if constexpr (P * sizeof(Real) % 16 == 0) {
+                span::regs_to_smem<Real, P>(win + lane * P, u);
+                span::regs_to_smem<Real, P>(win + 32 * P + lane * P, w);
+            } else {
 #pragma unroll
-            for (int i = 0; i < P; ++i) {
-                win[lane * P + i] = u[i];
-                win[32 * P + lane * P + i] = w[i];
+                for (int i = 0; i < P; ++i) {
+                    win[lane * P + i] = u[i];
+                    win[32 * P + lane * P + i] = w[i];
+                }
             }
         }
         __syncwarp();
