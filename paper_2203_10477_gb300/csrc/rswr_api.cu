@@ -376,35 +376,48 @@ rswr_status make_engine(Engine** out, int nprob, const rswr_problem* pr, int32_t
 
 // ---- pack / unpack between caller-packed arrays and the padded layout ----
 
-template <typename Real>
-__global__ void unpack_kernel(Real* state, const Real* packed, const int64_t* offsets, int nprob,
-                              const ProblemDev<Real>* problems, int64_t total)
+// PACK: packed <- state, else state <- packed, one component of a batch.  Bound by
+// HBM: a block moves 2048 consecutive packed points, eight loads of a thread in
+// flight, and looks its problem up once (a search per point, nine dependent loads,
+// held it to 1.4 TB/s: 392 us for 67 million FP32 points; the run that takes four
+// such copies went from 6871 to 5706 us); blocks that hold a problem's end walk
+// the offsets.
+template <typename Real, bool PACK>
+__global__ void __launch_bounds__(256) pack_kernel(Real* packed, Real* state, const int64_t* offsets, int nprob,
+                                                   const ProblemDev<Real>* problems, int64_t total)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    constexpr int K = 8, CH = 256 * K;
+    for (int64_t i0 = (int64_t)blockIdx.x * CH; i0 < total; i0 += (int64_t)gridDim.x * CH) {
         int lo = 0, hi = nprob - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (offsets[mid] <= i) lo = mid; else hi = mid - 1;
+            if (offsets[mid] <= i0) lo = mid; else hi = mid - 1;
         }
-        state[problems[lo].base + (i - offsets[lo])] = packed[i];
+        const int64_t i = i0 + threadIdx.x;
+        if (i0 + CH <= offsets[lo + 1]) {
+            const int64_t d = problems[lo].base - offsets[lo];
+            Real v[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[k] = PACK ? state[i + 256 * k + d] : packed[i + 256 * k];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                if (PACK) packed[i + 256 * k] = v[k];
+                else state[i + 256 * k + d] = v[k];
+            }
+        } else {
+            for (int k = 0; k < K; ++k) {
+                const int64_t j = i + 256 * k;
+                if (j >= total) break;
+                while (j >= offsets[lo + 1]) ++lo;
+                const int64_t at = problems[lo].base + (j - offsets[lo]);
+                if (PACK) packed[j] = state[at];
+                else state[at] = packed[j];
+            }
+        }
     }
 }
 
-template <typename Real>
-__global__ void pack_kernel(Real* packed, const Real* state, const int64_t* offsets, int nprob,
-                            const ProblemDev<Real>* problems, int64_t total)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nprob - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (offsets[mid] <= i) lo = mid; else hi = mid - 1;
-        }
-        packed[i] = state[problems[lo].base + (i - offsets[lo])];
-    }
-}
-
-int grid_for(int64_t n, int sms) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8)); }
+int grid_for(int64_t n, int sms) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, (int64_t)sms * 8)); }
 
 template <typename Real>
 rswr_status unpack(Engine* e, void* state, const void* packed, cudaStream_t s)
@@ -414,8 +427,8 @@ rswr_status unpack(Engine* e, void* state, const void* packed, cudaStream_t s)
                                   cudaMemcpyDeviceToDevice, s));
         return RSWR_OK;
     }
-    unpack_kernel<Real><<<grid_for(e->packed_len, e->num_sms), 256, 0, s>>>(
-        static_cast<Real*>(state), static_cast<const Real*>(packed), e->d_offsets, (int)e->probs.size(),
+    pack_kernel<Real, false><<<grid_for(e->packed_len, e->num_sms), 256, 0, s>>>(
+        static_cast<Real*>(const_cast<void*>(packed)), static_cast<Real*>(state), e->d_offsets, (int)e->probs.size(),
         static_cast<const ProblemDev<Real>*>(e->d_problems), e->packed_len);
     RSWR_CUDA(cudaGetLastError());
     return RSWR_OK;
@@ -429,8 +442,8 @@ rswr_status pack(Engine* e, void* packed, const void* state, cudaStream_t s)
                                   sizeof(Real) * e->probs[0].nx, cudaMemcpyDeviceToDevice, s));
         return RSWR_OK;
     }
-    pack_kernel<Real><<<grid_for(e->packed_len, e->num_sms), 256, 0, s>>>(
-        static_cast<Real*>(packed), static_cast<const Real*>(state), e->d_offsets, (int)e->probs.size(),
+    pack_kernel<Real, true><<<grid_for(e->packed_len, e->num_sms), 256, 0, s>>>(
+        static_cast<Real*>(packed), static_cast<Real*>(const_cast<void*>(state)), e->d_offsets, (int)e->probs.size(),
         static_cast<const ProblemDev<Real>*>(e->d_problems), e->packed_len);
     RSWR_CUDA(cudaGetLastError());
     return RSWR_OK;

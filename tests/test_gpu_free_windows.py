@@ -3,6 +3,8 @@ and probes where a warp's window begins and ends, on a lane's first and last
 registers, in halos only, two of them in one window, more probes than a warp
 records by itself; spans off and on the record buffer's eight levels; bit for bit
 against the CPU oracle on every such variant."""
+from types import SimpleNamespace
+
 import numpy as np
 import pytest
 
@@ -93,3 +95,26 @@ def test_passes_of_several_spans_equal_oracle(R, oracle_mod, ov):
     assert halos == [(m + 3) // 4 * 4 for m in (32 // S * S, S, 32 // S * S)]
     plan.set_span(S)
     assert plan.info()["halo"] == (S + 3) // 4 * 4
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_packing_of_uneven_problems(R, dtype):
+    """No step: the initial pair comes back, for problems shorter than, as long as and
+    longer than a block's 2048 points, with ends inside and on a block's edge."""
+    sizes = [64, 1984, 2048, 3, 2045, 40000, 65, 6144, 2047, 2049, 5, 100000]
+    probs = [SimpleNamespace(nx=n, xa=0.0, xb=1.0, a=1.0, dt=0.9 / (n - 1), n_sub=1, overlap=2) for n in sizes]
+    b = R.Batch(probs, dtype=dtype)
+    td = np.float64 if dtype else np.float32
+    r = inputs.rng(2)
+    q0, q1 = (r.standard_normal(sum(sizes)).astype(td) for _ in range(2))
+    f = r.standard_normal((len(sizes), 1)).astype(td)
+    got = b.run(f, f, 0, q0=q0, q1=q1)
+    u, w = q0.copy(), q1.copy()
+    at = 0
+    for n in sizes:
+        for j in (at, at + n - 1):
+            u[j] = f[sizes.index(n), 0]
+            w[j] = u[j] if dtype else 0
+        at += n
+    assert np.array_equal(got["u"].cpu().numpy(), u)
+    assert np.array_equal(got["w"].cpu().numpy(), w)
