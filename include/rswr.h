@@ -137,7 +137,7 @@ typedef struct rswr_plan_info {
     double c, c2, k, inv2dx;         /* double coefficients */
     float c2f, kf, inv2dxf;          /* F32 coefficients */
     int32_t span_steps;              /* S */
-    int32_t halo;                    /* H >= S: halo of a CTA window */
+    int32_t halo;                    /* H >= S: halo of a CTA window (the steps of a pass) */
     int32_t core;                    /* owned points per CTA tile */
     int32_t window;                  /* points per CTA window = core + 2H */
     int32_t points_per_thread, threads_per_cta, variant, mode;
@@ -151,7 +151,10 @@ typedef struct rswr_plan_info {
  * variant.  Errors: EINVAL for NULL arguments. */
 rswr_status rswr_plan_get_info(rswr_plan_t plan, rswr_plan_info* info);
 
-/* Steps per span, 1 <= S <= floor(overlap/2) (else EOVERLAP). */
+/* Steps per span, 1 <= S <= floor(overlap/2) (else EOVERLAP).  A span that was
+ * set is also what one launch or ticket advances; an FP32 plan as created
+ * (S = floor(overlap/2)) or tuned runs as many whole spans per pass as 32 steps
+ * hold.  The results are the same. */
 rswr_status rswr_plan_set_span(rswr_plan_t plan, int32_t S);
 
 /* Kernel variant (points per thread x threads per CTA) for the plan's dtype
@@ -306,8 +309,9 @@ rswr_status rswr_run_keep(rswr_plan_t plan, const void* fA, const void* fB, int6
  * from span-boundary states (the levels' Laplacians kept in shared memory,
  * or in tensor memory by the persistent FP32 sweep): by default every span
  * state is kept when they fit in half of the free device memory (one forward
- * sweep -- one resident launch when the plan's variant is a resident one and
- * its tiles fit -- then one persistent adjoint launch over all spans), else
+ * sweep, then one adjoint launch over all spans -- both on resident warps when
+ * the grid fits on the chip and the plan is as created or on a resident
+ * variant, else persistent), else
  * one checkpoint every ceil(sqrt(#spans)) spans with the states of each
  * segment recomputed before its spans are processed
  * (rswr_plan_set_checkpoint_spacing overrides).
@@ -457,9 +461,10 @@ rswr_status rswr_variant_get_tiling(int32_t v, int32_t* warp_halo, int32_t* wind
  *                                 moves the windows (tickets, TMA, flags);
  *   RSWR_VARIANT_RESIDENT         every warp keeps its window on chip for the
  *                                 whole run and only halo strips are exchanged,
- *                                 every so many spans; a grid that does not fit
- *                                 on the GPU at once is refused by rswr_run with
- *                                 RSWR_ENOTSUP.  A plan or batch as it was
+ *                                 every so many spans; a grid that is a little
+ *                                 too large runs on the default variant, one of
+ *                                 more than 13312 FP32 (3968 FP64) points per SM
+ *                                 is refused by rswr_run with RSWR_ENOTSUP.  A plan or batch as it was
  *                                 created runs this way by itself when it fits
  *                                 (same results); one whose variant, span or
  *                                 mode was set, or chosen by the autotuner,

@@ -1237,7 +1237,8 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
 // a resident one does, or takes the default variant where the grid is a little too
 // large (far too large: the run is refused); a plan as it was created
 // does when its grid fits on the chip; a variant, span or mode chosen by the
-// caller or the autotuner is kept to.
+// caller or the autotuner is kept to.  Every grid that fits is faster this way
+// (2x at 2^20 FP32 points, 9x at 8001; figures in resident.cuh).
 rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
 {
     *take = false;
