@@ -126,6 +126,7 @@ def span_roofline(dtype: str, value: float, ops: int, info: dict) -> dict:
     levels of its core out, once per span of S steps)."""
     w = 8 if dtype == "f64" else 4
     W, core, S = info["window"], info["core"], info["span_steps"]
+    S *= max(1, info["halo"] // S)  # a pass holds whole spans (its halo: its steps, rounded up to 4)
     bpu = w * (2 * W + 2 * core) / (core * S)
     hbm = load_peaks()["hbm_gbs"]
     alu = alu_roofline(dtype, value, ops)
