@@ -135,7 +135,8 @@ struct Engine {
     DevError* d_err = nullptr;
     void* d_host_stage = nullptr;  // rswr_run_host staging
     size_t host_stage_cap = 0;
-    void* d_scratch[2] = {nullptr, nullptr};  // adjoint scratch outputs
+    void* d_scratch[2] = {nullptr, nullptr};  // a packed state pair: the autotuner's outputs, and final states
+                                              // whose place a run still reads (scratch_pair)
     size_t scratch_cap = 0;
     cudaEvent_t ev_start = nullptr;  // caller-owned timing events (rswr_*_set_kernel_events)
     cudaEvent_t ev_stop = nullptr;
@@ -952,6 +953,71 @@ bool res_choose(Engine* e, int want_P, int S, int max_spans, bool sources, bool 
     return best->nw > 0;
 }
 
+// The engine's packed scratch pair (made at its first use, then kept).
+rswr_status scratch_pair(Engine* e)
+{
+    if (e->scratch_cap >= (size_t)e->packed_len) return RSWR_OK;
+    e->scratch_cap = 0;
+    for (int b = 0; b < 2; ++b) {
+        cudaFree(e->d_scratch[b]);
+        e->d_scratch[b] = nullptr;
+        if (cudaMalloc(&e->d_scratch[b], e->esize() * e->packed_len) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(RSWR_ENOMEM, "scratch");
+        }
+    }
+    e->scratch_cap = e->packed_len;
+    return RSWR_OK;
+}
+
+// A range of device memory (empty without an array).
+struct Range {
+    uintptr_t lo = 0, hi = 0;
+    Range(const void* p, size_t bytes) : lo((uintptr_t)p), hi(p ? (uintptr_t)p + bytes : (uintptr_t)p) {}
+    bool meets(const Range& o) const { return lo < o.hi && o.lo < hi; }
+};
+
+// What a probe writes.
+Range probe_range(const ProbeReq& q, size_t es)
+{
+    const int64_t last = q.stride * q.nmax * (int64_t)es;
+    return Range(static_cast<char*>(q.out) + std::min<int64_t>(last, 0), (size_t)std::llabs(last) + es);
+}
+
+// Whether the final state may not go straight to out0 / out1 while the run's
+// kernel still works: some of what it reads lies there (a run in place, say), or
+// another output of it, which the state replaces.
+bool outputs_meet(const Engine* e, const RunReq& r)
+{
+    const size_t es = e->esize(), state = es * (size_t)e->packed_len;
+    const size_t samples = es * e->probs.size() * (size_t)(r.T + 1);
+    int64_t rows = 0;
+    if (r.user_src)
+        for (const Engine::UserSrc& q : e->usrc) rows = std::max(rows, q.row + 1);
+    const Range reads[] = {Range(r.q0, state), Range(r.q0 ? r.q1 : nullptr, state), Range(r.fA, samples),
+                           Range(r.fB, samples), Range(e->usrc_samples, es * (size_t)(rows * e->usrc_pitch))};
+    const Range out[] = {Range(r.out0, state), Range(r.out1, state)};
+    if (out[0].meets(out[1])) return true;
+    for (const Range& o : out) {
+        for (const Range& x : reads)
+            if (o.meets(x)) return true;
+        for (const ProbeReq& q : r.probes)
+            if (o.meets(probe_range(q, es))) return true;
+    }
+    return false;
+}
+
+// Whether a probe's record lies in the initial state, which resident warps read
+// where the caller has it.
+bool probes_meet_state(const Engine* e, const RunReq& r)
+{
+    const size_t es = e->esize(), state = es * (size_t)e->packed_len;
+    if (r.q0)
+        for (const ProbeReq& q : r.probes)
+            if (probe_range(q, es).meets(Range(r.q0, state)) || probe_range(q, es).meets(Range(r.q1, state))) return true;
+    return false;
+}
+
 // States a resident run keeps for the adjoint sweep.
 struct ResKeep {
     void* ck0;
@@ -1036,6 +1102,10 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
     if (r.user_src && !e->usrc.empty() && e->usrc_pitch < r.T + 1)
         return fail(RSWR_EINVAL, "source samples hold fewer than T+1 levels");
+    // (a warp stores its points when its neighbours have loaded theirs at the
+    // earliest, and not even that in a run without an exchange)
+    const bool aside = outputs_meet(e, r);
+    if (aside && (st = scratch_pair(e)) != RSWR_OK) return st;
 
     // problems and warps
     std::vector<ResProb<Real>> probs(np);
@@ -1205,8 +1275,8 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     prm.srcs = reinterpret_cast<const ResSrc<Real>*>(t + b_prob + b_warp + b_probe);
     prm.in0 = static_cast<const Real*>(r.q0);
     prm.in1 = r.q0 ? static_cast<const Real*>(r.q1) : nullptr;
-    prm.out0 = static_cast<Real*>(r.out0);
-    prm.out1 = static_cast<Real*>(r.out1);
+    prm.out0 = static_cast<Real*>(aside && r.out0 ? e->d_scratch[0] : r.out0);
+    prm.out1 = static_cast<Real*>(aside && r.out1 ? e->d_scratch[1] : r.out1);
     if (keep) {
         prm.ck0 = static_cast<Real*>(keep->ck0);
         prm.ck1 = static_cast<Real*>(keep->ck1);
@@ -1230,6 +1300,9 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
     RSWR_CUDA(res_launch(e->dtype, e->form, rp.P, &prm, rp.grid, 32 * rp.per_cta, smem, rp.cluster, s));
     if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+    const size_t state = sizeof(Real) * (size_t)e->packed_len;
+    if (aside && r.out0) RSWR_CUDA(cudaMemcpyAsync(r.out0, e->d_scratch[0], state, cudaMemcpyDeviceToDevice, s));
+    if (aside && r.out1) RSWR_CUDA(cudaMemcpyAsync(r.out1, e->d_scratch[1], state, cudaMemcpyDeviceToDevice, s));
     return RSWR_OK;
 }
 
@@ -1245,6 +1318,7 @@ rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
     const VariantInfo vi = span_variant_info(e->variant);
     const bool sources = (r.user_src && !e->usrc.empty()) || (r.src && !r.js.empty());
     if (r.mono || r.from_state || r.steps_dev || r.T <= 0 || r.T >= ((int64_t)1 << 31) - 256) return RSWR_OK;
+    if (probes_meet_state(e, r)) return RSWR_OK;
     if (vi.resident) {
         *take = res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp);
         // (grids that a wider tiling of these variants once held still run, with tickets)
@@ -2255,15 +2329,8 @@ rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cu
             }
         }
     }
-    const size_t es = e->esize();
-    if (e->scratch_cap < (size_t)e->packed_len) {
-        for (int b = 0; b < 2; ++b) {
-            cudaFree(e->d_scratch[b]);
-            e->d_scratch[b] = nullptr;
-            if (cudaMalloc(&e->d_scratch[b], es * e->packed_len) != cudaSuccess) return fail(RSWR_ENOMEM, "scratch");
-        }
-        e->scratch_cap = e->packed_len;
-    }
+    rswr_status sp = scratch_pair(e);
+    if (sp != RSWR_OK) return sp;
     cudaEvent_t a, b;
     RSWR_CUDA(cudaEventCreate(&a));
     RSWR_CUDA(cudaEventCreate(&b));
@@ -2542,8 +2609,20 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             q.warp_values = rc.warp_values;
             pp.u = static_cast<Real*>(e->q0[0]) + ph.base;
             pp.w = static_cast<Real*>(e->q1[0]) + ph.base;
-            pp.uo = out0;
-            pp.wo = out1;
+            // (the last span's pieces are stored while others of it still read the samples)
+            RunReq io;
+            io.fA = fA;
+            io.fB = fB;
+            io.T = T;
+            io.out0 = out0;
+            io.out1 = out1;
+            const bool aside = outputs_meet(e, io);
+            if (aside) {
+                rswr_status st = scratch_pair(e);
+                if (st != RSWR_OK) return st;
+            }
+            pp.uo = aside ? static_cast<Real*>(e->d_scratch[0]) : out0;
+            pp.wo = aside ? static_cast<Real*>(e->d_scratch[1]) : out1;
             // both span words (bytes 0x7f: a value above any span), the grid barrier
             RSWR_CUDA(cudaMemsetAsync(d_span, 0x7f, 2 * sizeof(int), s));
             RSWR_CUDA(cudaMemsetAsync(d_span + 2, 0, sizeof(int), s));
@@ -2552,6 +2631,10 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
             RSWR_CUDA(paper_run_launch(rc, pp, q, e->num_sms, s));
             if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+            if (aside) {
+                RSWR_CUDA(cudaMemcpyAsync(out0, pp.uo, es * nx, cudaMemcpyDeviceToDevice, s));
+                RSWR_CUDA(cudaMemcpyAsync(out1, pp.wo, es * nx, cudaMemcpyDeviceToDevice, s));
+            }
             RSWR_CUDA(cudaMemcpyAsync(e->h_pstate, d_st, sizeof(PaperState), cudaMemcpyDeviceToHost, s));
             rswr_status st = check_engine(e, s, nullptr, nullptr, nullptr);
             if (st != RSWR_OK) return st;
