@@ -227,6 +227,14 @@ int default_variant(int dtype, int form, int S)
 // (re)allocates the state arrays when they grow.
 rswr_status layout(Engine* e)
 {
+    if (e->d_tiles) {
+        // a new tiling: runs queued so far still read the old one, and a captured
+        // graph holds its addresses (run_key does not)
+        RSWR_CUDA(cudaDeviceSynchronize());
+        if (e->graph_exec) cudaGraphExecDestroy(e->graph_exec);
+        e->graph_exec = nullptr;
+        e->graph_key.clear();
+    }
     const VariantInfo vi = span_variant_info(e->variant);
     e->P = vi.P;
     e->NT = vi.NT;

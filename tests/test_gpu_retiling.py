@@ -1,0 +1,84 @@
+"""Plans whose tiling changes between runs with the same arguments: a captured
+run is not replayed on the arrays of an earlier tiling, and a plan on a resident
+variant whose grid does not fit runs on a tiling of its own.  Bit for bit
+against the CPU oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2203_10477_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+F32, F64 = 0, 1
+
+
+@pytest.fixture(scope="module")
+def R():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2203_10477_gb300 import build, rswr
+
+    build.build()
+    return rswr
+
+
+class Call:
+    """The same tensors for every run, and the oracle's state."""
+
+    def __init__(self, oracle_mod, dtype, nx, T, cfl=0.9):
+        dt_ = np.float64 if dtype == F64 else np.float32
+        r = inputs.rng(nx)
+        self.dt, self.T = cfl / (nx - 1), T
+        fA, q0, q1 = (r.standard_normal(n).astype(dt_) for n in (T + 1, nx, nx))
+        kw = dict(form=0 if dtype == F64 else 1, prec="f64" if dtype == F64 else "f32")
+        ref = oracle_mod.leapfrog(nx, T, 1.0, self.dt, fA, np.zeros(T + 1, dt_), q0=q0, q1=q1, **kw)
+        dev = lambda x: torch.as_tensor(x, device="cuda")
+        self.fA, self.q0, self.q1, self.u, self.w = map(dev, (fA, q0, q1, ref["u"], ref["w"]))
+        self.out = (torch.empty_like(self.q0), torch.empty_like(self.q0))
+
+    def run(self, plan, what):
+        for o in self.out:
+            o.fill_(7.0)
+        plan.run(self.fA, None, self.T, q0=self.q0, q1=self.q1, out=self.out)
+        plan.check()
+        assert torch.equal(self.out[0], self.u) and torch.equal(self.out[1], self.w), what
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+def test_no_replay_after_a_new_tiling(R, oracle_mod, dtype):
+    nx = 300007
+    c = Call(oracle_mod, dtype, nx, 40)
+    plan = R.Plan(0.0, 1.0, 1.0, nx, c.dt, 16, 48, dtype=dtype)
+    own = [v for v in R.variants() if v["dtype"] == dtype and v["form"] == plan.info()["form"]]
+    S = plan.info()["span_steps"]
+    own = [v for v in own if v["max_span"] == 0 or v["max_span"] >= S]
+    tick = [v["variant"] for v in own if not v["resident"]]
+    plan.set_variant(tick[0])  # (off the resident path: runs are captured)
+    for rnd in range(2):
+        c.run(plan, f"{rnd}: captured")
+        c.run(plan, f"{rnd}: replayed")
+        # to a narrower tiling (more tiles: larger tables) and back
+        plan.set_variant(min(own, key=lambda v: v["window"])["variant"])
+        plan.set_variant(tick[0])
+        c.run(plan, f"{rnd}: after another variant")
+        plan.set_span(1)
+        plan.set_span(S)
+        c.run(plan, f"{rnd}: after another span")
+        plan.inject_missing_flag(0, 1 << 20)
+        plan.inject_missing_flag(-1, 0)
+        c.run(plan, f"{rnd}: after the hook was set and cleared")
+
+
+def test_no_replay_after_a_resident_variant_that_does_not_fit(R, oracle_mod):
+    nx = 1400003
+    c = Call(oracle_mod, F32, nx, 40)
+    plan = R.Plan(0.0, 1.0, 1.0, nx, c.dt, 64, 60, dtype=F32)
+    c.run(plan, "as created")
+    for v in [v["variant"] for v in R.variants() if v["dtype"] == F32 and v["resident"]]:
+        plan.set_variant(v)
+        c.run(plan, f"variant {v}")
+        c.run(plan, f"variant {v} again")
+    plan.set_variant(0)
+    c.run(plan, "the first variant again")
