@@ -95,6 +95,7 @@ struct Engine {
     int device = 0;
     int num_sms = 1;
     int variant = 0;
+    int tiling = 0;  // the variant that tickets and spans run on: `variant`, or the default one beside a resident variant
     int mode = RSWR_MODE_PERSISTENT;
     double wait_s = 5.0;
     int64_t ck_spacing = 0;  // adjoint checkpoint spacing in spans (0: automatic)
@@ -224,7 +225,9 @@ int default_variant(int dtype, int form, int S)
 }
 
 // Lays out tiles and padded problem regions for the current variant and S;
-// (re)allocates the state arrays when they grow.
+// (re)allocates the state arrays when they grow.  Resident windows need no tiles
+// (res_run cuts its own): beside such a variant the tiling is the default
+// variant's, for the runs that the resident kernel does not cover.
 rswr_status layout(Engine* e)
 {
     if (e->d_tiles) {
@@ -235,9 +238,13 @@ rswr_status layout(Engine* e)
         e->graph_exec = nullptr;
         e->graph_key.clear();
     }
-    const VariantInfo vi = span_variant_info(e->variant);
-    e->P = vi.P;
-    e->NT = vi.NT;
+    const VariantInfo vc = span_variant_info(e->variant);
+    e->P = vc.P;
+    e->NT = vc.NT;
+    if (!variant_takes_span(vc, e->S)) return fail(RSWR_EINVAL, "span longer than the warp halo of this variant");
+    e->tiling = vc.resident ? default_variant(e->dtype, e->form, e->S) : e->variant;
+    if (e->tiling < 0) return fail(RSWR_ENOTSUP, "no kernel variant runs this span");
+    const VariantInfo vi = span_variant_info(e->tiling);
     e->W = vi.W;
     // FP32 spans of 16 steps and fewer (overlaps below 64) are bound by the state's
     // way to memory and back: a pass of the span kernel takes as many whole spans
@@ -245,12 +252,11 @@ rswr_status layout(Engine* e)
     // caller chose the span.  512 uneven problems of overlap 32: 8382 -> 6871 us;
     // FP64 is bound by its pipe.
     int m = 1;
-    if (e->dtype == kF32 && !vi.resident && !e->span_set && e->inject_tile < 0)
+    if (e->dtype == kF32 && !e->span_set && e->inject_tile < 0)
         for (m = std::max(1, 32 / e->S); m > 1 && !variant_takes_span(vi, e->S * m);) --m;
     e->pass = e->S * m;
     e->H = (e->pass + 3) / 4 * 4;
     e->core = e->W - 2 * e->H;
-    if (!variant_takes_span(vi, e->S)) return fail(RSWR_EINVAL, "span longer than the warp halo of this variant");
     if (e->core < e->H || e->core < 4) return fail(RSWR_EINVAL, "span too long for the CTA window of this variant");
     const int64_t pad = e->H + 8;
     int64_t at = 0, tile = 0, off = 0;
@@ -728,19 +734,19 @@ rswr_status device_work(Engine* e, const RunReq& r, int nprobe, int64_t mono_blk
         SpanParams<Real> prm = span_params<Real>(e, r.T, nspans);
         prm.steps_dev = r.steps_dev;
         int bps = 0;
-        RSWR_CUDA(span_occupancy(e->variant, &bps));
+        RSWR_CUDA(span_occupancy(e->tiling, &bps));
         if (bps < 1) return fail(RSWR_ENOTSUP, "span kernel does not fit on an SM");
         if (nspans > 0) {
             if (e->mode == RSWR_MODE_PERSISTENT) {
                 RSWR_CUDA(cudaMemsetAsync(e->d_ticket, 0, sizeof(unsigned long long), s));
                 RSWR_CUDA(cudaMemsetAsync(e->d_done, 0, sizeof(int) * e->ntiles, s));
                 const int grid = (int)std::min<int64_t>((int64_t)bps * e->num_sms, (int64_t)nspans * e->ntiles);
-                RSWR_CUDA(span_launch(e->variant, &prm, grid, s));
+                RSWR_CUDA(span_launch(e->tiling, &prm, grid, s));
             } else {
                 const int grid = (int)std::min<int64_t>((int64_t)bps * e->num_sms, e->ntiles);
                 for (int k = 0; k < nspans; ++k) {
                     prm.span = k;
-                    RSWR_CUDA(span_launch(e->variant, &prm, grid, s));
+                    RSWR_CUDA(span_launch(e->tiling, &prm, grid, s));
                 }
             }
         }
@@ -803,7 +809,7 @@ std::vector<int64_t> run_key(const Engine* e, const RunReq& r)
 {
     auto P = [](const void* p) { return (int64_t)(intptr_t)p; };
     std::vector<int64_t> k{r.mono, P(r.fA), P(r.fB), r.T, P(r.q0), P(r.q1), P(r.out0), P(r.out1), P(r.src),
-                           r.src_pitch, r.src_stride, e->variant, e->mode, e->S, e->H, P(e->ev_start),
+                           r.src_pitch, r.src_stride, e->tiling, e->mode, e->S, e->H, P(e->ev_start),
                            P(e->ev_stop), e->inject_tile, e->inject_span, (int64_t)(e->wait_s * 1e3),
                            (int64_t)r.probes.size(), r.user_src ? (int64_t)e->usrc.size() : -1, P(e->d_srcs),
                            e->srcs_live};
@@ -874,7 +880,8 @@ double res_cost(int dtype, int P, int S, int warps_per_sm, bool linked, bool clu
 // The best cut with P points per lane (P = 0: over all compiled P); false when
 // the grid does not fit on the GPU at once.  An exchange follows every m spans
 // of S steps, H = m S halo points wide (the Theorem's bound for the windows).
-bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources, bool probes, bool kept, ResPlan* best)
+// slack: windows with room to put a source or probe on an end register.
+bool res_search(const Engine* e, int want_P, int S, int max_spans, bool slack, bool probes, bool kept, ResPlan* best)
 {
     static const int Pf[] = {4, 8, 16, 32}, Pd[] = {1, 2, 4, 8, 12, 16};
     const int* Ps = e->dtype == kF64 ? Pd : Pf;
@@ -890,7 +897,7 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool sources,
             r.P = P;
             r.S = H;
             r.H = H;
-            r.slack = (sources || probes) && res_own(P, H, true) >= 2 * H + 2;
+            r.slack = slack && res_own(P, H, true) >= 2 * H + 2;
             // (kept states want pieces on multiples of four points: 16-byte stores)
             const int own = r.own = res_own(P, H, r.slack) - (kept ? 4 : 0);
             if (own < 4) break;
@@ -954,7 +961,12 @@ bool res_choose(Engine* e, int want_P, int S, int max_spans, bool sources, bool 
     auto it = e->res_plans.find(key);
     if (it == e->res_plans.end()) {
         ResPlan r;
-        if (!res_search(e, want_P, S, max_spans, sources, probes, kept, &r)) r.nw = 0;
+        // (no cut with that room fits, 1.13 to 1.17 million FP32 points on 152 SMs: the
+        // slower ways of the windows with a source or probe still beat tickets)
+        const bool slack = sources || probes;
+        if (!res_search(e, want_P, S, max_spans, slack, probes, kept, &r) &&
+            !(slack && res_search(e, want_P, S, max_spans, false, probes, kept, &r)))
+            r.nw = 0;
         it = e->res_plans.emplace(key, r).first;
     }
     *best = it->second;
@@ -1314,8 +1326,12 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     return RSWR_OK;
 }
 
+// Points per SM (FP32, FP64) beyond which a plan that asked for a resident variant
+// is told so instead of being run with tickets: include/rswr.h promises these.
+constexpr int64_t kResRefused[] = {13312, 3968};
+
 // Whether a run takes the resident path, and its cut.  A plan whose variant is
-// a resident one does, or takes the default variant where the grid is a little too
+// a resident one does, or runs with tickets where the grid is a little too
 // large (far too large: the run is refused); a plan as it was created
 // does when its grid fits on the chip; a variant, span or mode chosen by the
 // caller or the autotuner is kept to.  Every grid that fits is faster this way
@@ -1329,37 +1345,13 @@ rswr_status res_route(Engine* e, const RunReq& r, bool* take, ResPlan* rp)
     if (probes_meet_state(e, r)) return RSWR_OK;
     if (vi.resident) {
         *take = res_choose(e, vi.P, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp);
-        // (grids that a wider tiling of these variants once held still run, with tickets)
-        const int64_t most = (int64_t)e->num_sms * (e->dtype == kF32 ? 13312 : 3968);
-        if (!*take && (e->packed_len > most || e->inject_tile >= 0))
+        if (!*take && (e->packed_len > (int64_t)e->num_sms * kResRefused[e->dtype] || e->inject_tile >= 0))
             return fail(RSWR_ENOTSUP, "resident variant: the grid does not fit on the GPU at once");
     } else if (!e->chosen && e->mode == RSWR_MODE_PERSISTENT && e->inject_tile < 0) {
         *take = res_choose(e, 0, e->S, kResMaxHalo, sources, !r.probes.empty(), false, rp);
     }
     return RSWR_OK;
 }
-
-// A plan on a resident variant takes the default variant for a run that the
-// resident kernel does not cover, and its own tiling back afterwards.
-struct Ticketed {
-    Engine* e;
-    int variant;
-    rswr_status st = RSWR_OK;
-    Ticketed(Engine* e_, bool needed) : e(e_), variant(-1)
-    {
-        if (!needed || !span_variant_info(e->variant).resident) return;
-        variant = e->variant;
-        e->variant = default_variant(e->dtype, e->form, e->S);
-        st = layout(e);
-    }
-    ~Ticketed()
-    {
-        if (variant < 0) return;
-        cudaDeviceSynchronize();  // the run still reads the tiling that goes
-        e->variant = variant;
-        layout(e);
-    }
-};
 
 template <typename Real>
 rswr_status run_impl(Engine* e, const RunReq& r, cudaStream_t s)
@@ -1369,8 +1361,6 @@ rswr_status run_impl(Engine* e, const RunReq& r, cudaStream_t s)
     rswr_status st = res_route(e, r, &res, &rp);
     if (st != RSWR_OK) return st;
     if (res) return res_run<Real>(e, r, rp, nullptr, s);
-    Ticketed ticketed(e, !r.mono && r.T > 0);
-    if (ticketed.st != RSWR_OK) return ticketed.st;
     int nprobe = 0;
     int64_t mono_blk_off = -1;
     st = prepare_tables<Real>(e, r, &nprobe, &mono_blk_off, s);
@@ -2457,8 +2447,6 @@ template <typename Real>
 rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, const Real* q0, const Real* q1, Real* out0,
                       Real* out1, int64_t* spans, int64_t spans_cap, int64_t* nspans, double beta, cudaStream_t s)
 {
-    Ticketed ticketed(e, true);  // the spans continue from the state arrays
-    if (ticketed.st != RSWR_OK) return ticketed.st;
     const ProbHost& ph = e->probs[0];
     const int64_t nx = ph.nx, N = ph.n_sub, ov = ph.ov, el = (ov + 1) / 2, er = ov / 2;
     const size_t es = sizeof(Real);

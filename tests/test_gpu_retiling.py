@@ -82,3 +82,55 @@ def test_no_replay_after_a_resident_variant_that_does_not_fit(R, oracle_mod):
         c.run(plan, f"variant {v} again")
     plan.set_variant(0)
     c.run(plan, "the first variant again")
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+def test_resident_variant_runs_what_its_kernel_does_not_cover(R, oracle_mod, dtype):
+    """A plan on a resident variant: spans longer than its windows take (FP64),
+    probes over the initial state, a continued paper-literal run, and the plan's
+    own runs between them, on one tiling that stays."""
+    import ctypes
+
+    nx, T, jr = 30011, 150, 15000
+    c = Call(oracle_mod, dtype, nx, T)
+    ov = 64 if dtype == F32 else 160
+    plan = R.Plan(0.0, 1.0, 1.0, nx, c.dt, 3, ov, dtype=dtype)
+    tiles = plan.info()["ntiles"]
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    ref = plan.run(c.fA, None, T, q0=c.q0, q1=c.q1, j_r=jr)["recv"]
+    paper = plan.run_paper(c.fA, None, T, q0=c.q0, q1=c.q1)
+    for v in [v for v in R.variants() if v["dtype"] == dtype and v["resident"] and v["max_span"] >= ov // 2]:
+        plan.set_variant(v["variant"])
+        assert plan.info()["variant"] == v["variant"] and plan.info()["ntiles"] == tiles
+        c.run(plan, v)
+        u = c.q0.clone()
+        rec = u[jr:jr + T + 1]
+        R.check(R.lib().rswr_run(plan.h, p(c.fA), None, T, p(u), p(c.q1), p(c.out[0]), p(c.out[1]), None, jr, p(rec),
+                                 torch.cuda.current_stream().cuda_stream))
+        plan.check()
+        assert torch.equal(rec, ref) and torch.equal(c.out[0], c.u), v
+        got = plan.run_paper(c.fA, None, T, q0=c.q0, q1=c.q1)
+        assert torch.equal(got["u"], paper["u"]) and list(got["spans"]) == list(paper["spans"]), v
+        c.run(plan, v)
+
+
+def test_grids_whose_windows_have_no_room_to_shift(R, oracle_mod):
+    """Windows that fit the chip only without room to put a source or a probe on
+    an end register."""
+    nx, T = 1150001, 70
+    c = Call(oracle_mod, F32, nx, T)
+    plan = R.Plan(0.0, 1.0, 1.0, nx, c.dt, 64, 64, dtype=F32)
+    c.run(plan, "nothing special")
+    js = [1, 333333, nx // 2, nx - 2]
+    s = inputs.rng(3).standard_normal((len(js), T + 1)).astype(np.float32)
+    h = lambda t: t.cpu().numpy()
+    for src in (None, js):
+        plan.set_sources(src, s if src else None)
+        kw = dict(src_j=np.asarray(js, np.int64), src=s) if src else {}
+        ref = oracle_mod.leapfrog(nx, T, 1.0, c.dt, h(c.fA), np.zeros(T + 1, np.float32), q0=h(c.q0), q1=h(c.q1), form=1,
+                                  prec="f32", rec_j=[0, 1, 333330, 333333, nx // 2 + 1, nx - 2, nx - 1], **kw)
+        for i, jr in enumerate([0, 1, 333330, 333333, nx // 2 + 1, nx - 2, nx - 1]):
+            got = plan.run(c.fA, None, T, q0=c.q0, q1=c.q1, j_r=jr)
+            plan.check()
+            assert np.array_equal(h(got["recv"]), ref["rec"][i]), (src, jr)
+        assert np.array_equal(h(got["u"]), ref["u"]) and np.array_equal(h(got["w"]), ref["w"]), src
