@@ -39,7 +39,6 @@ rswr_status fail(rswr_status st, const std::string& m)
             return fail(RSWR_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_));           \
     } while (0)
 
-constexpr int kSpanCap = 256;     // largest span a CTA window supports
 constexpr int64_t kAlign = 32;    // every problem region starts on a 32-element boundary
 
 struct ProbHost {

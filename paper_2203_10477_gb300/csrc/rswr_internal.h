@@ -13,6 +13,8 @@ namespace rswr {
 enum Form : int { kCanonical = 0, kIncrement = 1 };
 enum DType : int { kF32 = 0, kF64 = 1 };
 
+constexpr int kSpanCap = 256;  // largest span a CTA window supports
+
 // One independent 1-D problem inside a plan or a batch.  Grid point j of the
 // problem lives at index base + j of every state array; the arrays are padded
 // with at least H zero points on both sides of every problem.

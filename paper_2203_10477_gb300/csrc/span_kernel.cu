@@ -46,12 +46,14 @@ Entry make_entry_WS()
 }
 
 // resident warp windows (resident_kernel.cu launches them): a window holds its
-// halos and more points of its own than they, so spans of fewer than 8 P steps
+// halos and more points of its own than they, so spans of fewer than 8 P steps.
+// An FP64 plan may set longer ones all the same, which run with tickets.
 template <typename Real, int FORM, int P, int NT, int KH, int MINB>
 Entry make_entry_RES()
 {
     Entry e;
-    const int max_span = 8 * P - 2 < kResMaxHalo ? 8 * P - 2 : kResMaxHalo;
+    const int longest = 8 * P - 2 < kResMaxHalo ? 8 * P - 2 : kResMaxHalo;
+    const int max_span = sizeof(Real) == 8 ? kSpanCap : longest;
     e.info = VariantInfo{sizeof(Real) == 8 ? kF64 : kF32, FORM, P, NT, KH, 32 * P, NT, max_span, 1};
     e.fn = nullptr;
     e.fn_src = nullptr;

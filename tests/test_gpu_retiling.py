@@ -99,7 +99,9 @@ def test_resident_variant_runs_what_its_kernel_does_not_cover(R, oracle_mod, dty
     p = lambda t: ctypes.c_void_p(t.data_ptr())
     ref = plan.run(c.fA, None, T, q0=c.q0, q1=c.q1, j_r=jr)["recv"]
     paper = plan.run_paper(c.fA, None, T, q0=c.q0, q1=c.q1)
-    for v in [v for v in R.variants() if v["dtype"] == dtype and v["resident"] and v["max_span"] >= ov // 2]:
+    todo = [v for v in R.variants() if v["dtype"] == dtype and v["resident"] and v["max_span"] >= ov // 2]
+    assert todo
+    for v in todo:
         plan.set_variant(v["variant"])
         assert plan.info()["variant"] == v["variant"] and plan.info()["ntiles"] == tiles
         c.run(plan, v)
@@ -134,3 +136,18 @@ def test_grids_whose_windows_have_no_room_to_shift(R, oracle_mod):
             plan.check()
             assert np.array_equal(h(got["recv"]), ref["rec"][i]), (src, jr)
         assert np.array_equal(h(got["u"]), ref["u"]) and np.array_equal(h(got["w"]), ref["w"]), src
+
+
+def test_fp64_resident_variants_take_every_span(R, oracle_mod):
+    """Spans of up to 256 steps are accepted whether the variant or the span comes
+    first."""
+    nx = 9001
+    c = Call(oracle_mod, F64, nx, 300)
+    for v in [v["variant"] for v in R.variants() if v["dtype"] == F64 and v["resident"]]:
+        plan = R.Plan(0.0, 1.0, 1.0, nx, c.dt, 2, 512, dtype=F64)
+        assert plan.info()["span_steps"] == 256
+        plan.set_variant(v)
+        for S in (256, 63, 200):
+            plan.set_span(S)
+            assert plan.info()["variant"] == v and plan.info()["span_steps"] == S
+            c.run(plan, (v, S))
