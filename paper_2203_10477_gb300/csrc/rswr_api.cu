@@ -697,6 +697,18 @@ rswr_status prepare_tables(Engine* e, const RunReq& r, int* nprobe, int64_t* mon
     return RSWR_OK;
 }
 
+// Records a caller's timing event: in a captured run as a node that records it
+// at every replay (a plain stream refuses that form).
+rswr_status record_event(cudaEvent_t ev, cudaStream_t s)
+{
+    if (!ev) return RSWR_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    RSWR_CUDA(cudaStreamIsCapturing(s, &cap));
+    RSWR_CUDA(cudaEventRecordWithFlags(ev, s, cap == cudaStreamCaptureStatusNone ? cudaEventRecordDefault
+                                                                                 : cudaEventRecordExternal));
+    return RSWR_OK;
+}
+
 // The device work of one run (capturable in a CUDA graph: no host sync, no
 // host-to-device copies).
 template <typename Real>
@@ -727,7 +739,7 @@ rswr_status device_work(Engine* e, const RunReq& r, int nprobe, int64_t mono_blk
 
     const void* fin0;
     const void* fin1;
-    if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
+    if ((st = record_event(e->ev_start, s)) != RSWR_OK) return st;
     if (!r.mono) {
         const int nspans = (int)((r.T + e->pass - 1) / e->pass);
         SpanParams<Real> prm = span_params<Real>(e, r.T, nspans);
@@ -796,7 +808,7 @@ rswr_status device_work(Engine* e, const RunReq& r, int nprobe, int64_t mono_blk
             fin1 = b;
         }
     }
-    if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+    if ((st = record_event(e->ev_stop, s)) != RSWR_OK) return st;
     RSWR_CUDA(probe_final_launch(e->dtype, e->d_probes, nprobe, fin0, r.T, s));
     if (r.out0 && (st = pack<Real>(e, r.out0, fin0, s)) != RSWR_OK) return st;
     if (r.out1 && (st = pack<Real>(e, r.out1, fin1, s)) != RSWR_OK) return st;
@@ -1316,9 +1328,10 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     int values = 0;
     const size_t smem = res_smem_bytes(e->dtype, rp.P, rp.H, rp.per_cta, r.probes.empty() ? 0 : 2, &values);
     prm.x = res_exchange(e, rp.H, values, rp.cluster);
-    if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
+    // (the events time runs, not a gradient's own forward sweep)
+    if (!keep && (st = record_event(e->ev_start, s)) != RSWR_OK) return st;
     RSWR_CUDA(res_launch(e->dtype, e->form, rp.P, &prm, rp.grid, 32 * rp.per_cta, smem, rp.cluster, s));
-    if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+    if (!keep && (st = record_event(e->ev_stop, s)) != RSWR_OK) return st;
     const size_t state = sizeof(Real) * (size_t)e->packed_len;
     if (aside && r.out0) RSWR_CUDA(cudaMemcpyAsync(r.out0, e->d_scratch[0], state, cudaMemcpyDeviceToDevice, s));
     if (aside && r.out1) RSWR_CUDA(cudaMemcpyAsync(r.out1, e->d_scratch[1], state, cudaMemcpyDeviceToDevice, s));
@@ -2529,13 +2542,20 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
     // level 0 (paper Sec. 2.1, or the given state) in the plan's own state
     // arrays; the runs below continue from there (no graph capture: the span
     // kernel's arguments change every span)
-    const bool keep_graph = e->use_graph;
-    e->use_graph = false;
+    // (and the timing events bracket all of its kernels)
     struct Restore {
         Engine* e;
         bool g;
-        ~Restore() { e->use_graph = g; }
-    } restore{e, keep_graph};
+        cudaEvent_t a, b;
+        ~Restore()
+        {
+            e->use_graph = g;
+            e->ev_start = a;
+            e->ev_stop = b;
+        }
+    } restore{e, e->use_graph, e->ev_start, e->ev_stop};
+    e->use_graph = false;
+    e->ev_start = e->ev_stop = nullptr;
     {
         RunReq r;
         r.fA = fA;
@@ -2623,16 +2643,16 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             RSWR_CUDA(cudaMemsetAsync(d_span + 2, 0, sizeof(int), s));
             RSWR_CUDA(cudaMemcpyAsync(d_pieces, pieces.data(), sizeof(PaperPiece) * pieces.size(),
                                       cudaMemcpyHostToDevice, s));
-            if (e->ev_start) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_start, s, cudaEventRecordExternal));
+            rswr_status st = record_event(restore.a, s);
+            if (st != RSWR_OK) return st;
             RSWR_CUDA(paper_run_launch(rc, pp, q, e->num_sms, s));
-            if (e->ev_stop) RSWR_CUDA(cudaEventRecordWithFlags(e->ev_stop, s, cudaEventRecordExternal));
+            if ((st = record_event(restore.b, s)) != RSWR_OK) return st;
             if (aside) {
                 RSWR_CUDA(cudaMemcpyAsync(out0, pp.uo, es * nx, cudaMemcpyDeviceToDevice, s));
                 RSWR_CUDA(cudaMemcpyAsync(out1, pp.wo, es * nx, cudaMemcpyDeviceToDevice, s));
             }
             RSWR_CUDA(cudaMemcpyAsync(e->h_pstate, d_st, sizeof(PaperState), cudaMemcpyDeviceToHost, s));
-            rswr_status st = check_engine(e, s, nullptr, nullptr, nullptr);
-            if (st != RSWR_OK) return st;
+            if ((st = check_engine(e, s, nullptr, nullptr, nullptr)) != RSWR_OK) return st;
             const int64_t taken = e->h_pstate->count;
             if (spans && taken > 0)
                 RSWR_CUDA(cudaMemcpy(spans, d_rec, sizeof(int64_t) * (size_t)std::min<int64_t>(taken, rec_cap),
@@ -2646,6 +2666,8 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
     const size_t smem_i = es * (8 * (size_t)(ov + tau_max + 2)) + sizeof(int) * (size_t)(ov + 2);
     const size_t smem_r = es * 4 * (size_t)(CH + 2 * cap + 2);
     int64_t n0 = 0, m_count = 0;
+    rswr_status rec = record_event(restore.a, s);
+    if (rec != RSWR_OK) return rec;
     while (n0 < T) {
         // as many spans as the run needs at least (each advances at most cap
         // levels), so the batch never runs past T; then one read-back
@@ -2693,6 +2715,7 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             return fail(RSWR_ECUDA, "paper-literal run made no progress");
         }
     }
+    if ((rec = record_event(restore.b, s)) != RSWR_OK) return rec;
     if (spans && m_count > 0)
         RSWR_CUDA(cudaMemcpyAsync(spans, d_rec, sizeof(int64_t) * (size_t)std::min<int64_t>(m_count, rec_cap),
                                   cudaMemcpyDeviceToHost, s));
