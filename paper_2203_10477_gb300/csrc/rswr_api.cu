@@ -131,7 +131,7 @@ struct Engine {
     std::vector<unsigned char> res_tables;
     uint32_t res_epoch = 0;
     std::map<std::vector<int>, ResPlan> res_plans;
-    bool chosen = false;  // variant or span set by the caller or the autotuner: runs keep to them
+    bool chosen = false;  // variant, span or mode set by the caller or the autotuner: runs keep to them
     DevError* d_err = nullptr;
     void* d_host_stage = nullptr;  // rswr_run_host staging
     size_t host_stage_cap = 0;
@@ -2860,6 +2860,7 @@ rswr_status rswr_plan_set_mode(rswr_plan_t plan, int32_t mode)
     if (!plan) return fail(RSWR_EINVAL, "NULL plan");
     if (mode != RSWR_MODE_PERSISTENT && mode != RSWR_MODE_PER_SPAN) return fail(RSWR_EINVAL, "bad mode");
     plan->e->mode = mode;
+    plan->e->chosen = true;
     return RSWR_OK;
 }
 
@@ -3064,6 +3065,7 @@ rswr_status rswr_batch_set_mode(rswr_batch_t batch, int32_t mode)
     if (!batch) return fail(RSWR_EINVAL, "NULL batch");
     if (mode != RSWR_MODE_PERSISTENT && mode != RSWR_MODE_PER_SPAN) return fail(RSWR_EINVAL, "bad mode");
     batch->e->mode = mode;
+    batch->e->chosen = true;
     return RSWR_OK;
 }
 
