@@ -205,9 +205,8 @@ __global__ void __launch_bounds__(32 * radj_max_warps<Real>(P), 1)
         int n0, len;
         levels(prm.parts - 1, n0, len);
         ask(n0, len);
-        // FP32: the spans' sums in two floats (an exact sum and its remainder; a
-        // double addition takes 64 clocks of the pipe per warp), FP64: as they are
-        Real acc = Real(0), acc_lo = Real(0);
+        // (a span's sums meet in double: the sum over the spans may leave FP32's range)
+        double acc = 0.0;
         constexpr int G = sizeof(Real) == 4 && P > 8 ? P / 8 : 1;  // summation groups of a lane
         Real racc[G];
 #pragma unroll
@@ -501,14 +500,7 @@ __global__ void __launch_bounds__(32 * radj_max_warps<Real>(P), 1)
             if (span_done) {
 #pragma unroll
                 for (int q = 0; q < G; ++q) {
-                    const Real x1 = owner ? racc[q] : Real(0);
-                    if constexpr (sizeof(Real) == 4) {
-                        const Real t = radd(acc, x1), y = rsub(t, acc);
-                        acc_lo = radd(acc_lo, radd(rsub(acc, rsub(t, y)), rsub(x1, y)));
-                        acc = t;
-                    } else {
-                        acc = radd(acc, x1);
-                    }
+                    acc += owner ? (double)racc[q] : 0.0;
                     racc[q] = Real(0);
                 }
             }
@@ -536,7 +528,7 @@ __global__ void __launch_bounds__(32 * radj_max_warps<Real>(P), 1)
             n0 = n0_next;
             len = len_next;
         }
-        double sum = (double)acc + (double)acc_lo;
+        double sum = acc;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(kFull, sum, o);
         if (lane == 0) prm.sums[g] = sum;

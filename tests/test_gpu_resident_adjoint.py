@@ -1,0 +1,48 @@
+"""The gradient with dL/da on resident windows (csrc/resident_adjoint.cu)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2203_10477_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+F32, F64 = 0, 1
+
+
+@pytest.fixture(scope="module")
+def R():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2203_10477_gb300 import build, rswr
+
+    build.build()
+    return rswr
+
+
+@pytest.mark.parametrize("nx", [5001, 1 << 20])  # eight and sixteen points per lane
+def test_sums_over_spans_leave_fp32s_range(R, oracle_mod, nx):
+    """With a cotangent of 2^112 a chain of products (eight points, one span) stays
+    below FP32's largest value: at most 7.5e3 times 2^112, while the sum of a
+    point's chains over all spans is 5.6e5 times 2^112, beyond it (both from the
+    same sweeps in FP64; nothing returns from the grid's right end).  The resident
+    sweep against the persistent one (a plan on a variant with tickets), which
+    sums its spans in double: the same chains, or chains of at most 128 terms that
+    meet in another order."""
+    T, jr = 4000, 300
+    t = np.arange(T + 1)
+    fA = (1e5 * np.sin(np.pi * t / T) ** 2).astype(np.float32)
+    wbar = np.full(T + 1, 2.0 ** 112, np.float32)
+    got = []
+    for variant in (None, 0):
+        plan = R.Plan(0.0, 1.0, 1.0, nx, 0.9 / (nx - 1), 8, 64, dtype=F32)
+        if variant is not None:
+            plan.set_variant(variant)
+        got.append(plan.adjoint(fA, None, T, jr, wbar, want_a=True))
+        plan.check()
+    da = [g["grad_a"].item() for g in got]
+    ref = oracle_mod.adjoint(5001, T, 1.0, 0.9 / 5000, fA, np.zeros(T + 1), jr, np.ones(T + 1))
+    assert all(abs(x) > 2.0 ** 128 for x in da)
+    assert abs(da[0] - da[1]) * 2.0 ** -112 <= 128 * 2.0 ** -24 * ref["abs_da"], da
+    assert torch.equal(got[0]["grad_fA"], got[1]["grad_fA"])
