@@ -194,7 +194,8 @@ rswr_status rswr_plan_set_sources(rswr_plan_t plan, int64_t nsrc, const int64_t*
 
 /* Failure-injection hook for tests: in persistent mode, CTA tile `tile` does
  * not publish completion of span `span`, so its neighbours' bounded waits
- * expire and the run reports RSWR_ETIMEOUT.  tile = -1 disables. */
+ * expire and the run reports RSWR_ETIMEOUT.  Gradients run without it.
+ * tile = -1 disables. */
 rswr_status rswr_plan_inject_missing_flag(rswr_plan_t plan, int32_t tile, int32_t span);
 
 /* Timing hook: when set, every run records `start` (a cudaEvent_t passed as

@@ -1323,7 +1323,7 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     // uses up: one more exchange before the last level is recorded
     if (!r.probes.empty() && steps % rp.S == 0) prm.nchunks += 1;
     prm.nwarps = (int32_t)warps.size();
-    prm.inject_warp = e->inject_tile;
+    prm.inject_warp = keep ? -1 : e->inject_tile;  // (gradients run without the hook)
     prm.inject_chunk = (int32_t)((int64_t)e->inject_span * e->S / rp.S);
     int values = 0;
     const size_t smem = res_smem_bytes(e->dtype, rp.P, rp.H, rp.per_cta, r.probes.empty() ? 0 : 2, &values);

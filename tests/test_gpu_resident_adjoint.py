@@ -46,3 +46,35 @@ def test_sums_over_spans_leave_fp32s_range(R, oracle_mod, nx):
     assert all(abs(x) > 2.0 ** 128 for x in da)
     assert abs(da[0] - da[1]) * 2.0 ** -112 <= 128 * 2.0 ** -24 * ref["abs_da"], da
     assert torch.equal(got[0]["grad_fA"], got[1]["grad_fA"])
+
+
+
+def gradient(R, dtype, nx, T=300, jr=200):
+    td = torch.float64 if dtype == F64 else torch.float32
+    fA, w = (torch.as_tensor(inputs.rng(s).standard_normal(T + 1), device="cuda").to(td) for s in (1, 2))
+    plan = R.Plan(0.0, 1.0, 1.3, nx, 0.9 / (nx - 1) / 1.3, 8, 64, dtype=dtype)
+
+    def grad():
+        g = plan.adjoint(fA, None, T, jr, w, want_a=True)
+        return g["grad_fA"].clone(), g["grad_a"].clone()
+
+    return plan, grad, lambda: plan.run_keep(fA, None, T, j_r=jr)
+
+
+def same(a, b):
+    return all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+def test_gradients_run_without_the_hook(R, dtype):
+    plan, grad, keep = gradient(R, dtype, 20001)
+    ref, kept = grad(), keep()
+    plan.set_wait_limit(0.2)
+    for tile, span in ((1, 0), (2, 3)):
+        plan.inject_missing_flag(tile, span)
+        got = grad()
+        plan.check()
+        assert same(got, ref)
+        again = keep()
+        plan.check()
+        assert torch.equal(again["u"], kept["u"]) and torch.equal(again["recv"], kept["recv"])
