@@ -194,8 +194,12 @@ rswr_status rswr_plan_set_sources(rswr_plan_t plan, int64_t nsrc, const int64_t*
 
 /* Failure-injection hook for tests: in persistent mode, CTA tile `tile` does
  * not publish completion of span `span`, so its neighbours' bounded waits
- * expire and the run reports RSWR_ETIMEOUT.  Gradients run without it.
+ * expire and the run reports RSWR_ETIMEOUT.  Gradients run without it.  With
+ * span = RSWR_INJECT_SWEEP + m it is runs that go without, and the m-th exchange of
+ * a resident gradient's adjoint sweep (warp `tile`) or grid barrier of a
+ * paper-literal run in one launch (CTA `tile`) that is not published.
  * tile = -1 disables. */
+#define RSWR_INJECT_SWEEP 0x40000000
 rswr_status rswr_plan_inject_missing_flag(rswr_plan_t plan, int32_t tile, int32_t span);
 
 /* Timing hook: when set, every run records `start` (a cudaEvent_t passed as

@@ -573,12 +573,14 @@ __global__ void __launch_bounds__(32 * kRunWarps, 4) paper_run_kernel(const __gr
     const int64_t gw = (int64_t)warp * gridDim.x + blockIdx.x, nw = (int64_t)gridDim.x * kRunWarps;
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned target = 0;
+    int barriers = 0;
     auto barrier = [&](int count, int side) {
         target += gridDim.x;
         __syncthreads();
+        const int no = barriers++;
         if (threadIdx.x == 0) {
             __threadfence();
-            atomicAdd(q.arrived, 1u);
+            if ((int)blockIdx.x != q.inject_cta || no < q.inject_barrier) atomicAdd(q.arrived, 1u);
             long long t0 = 0;
             int ok = 1;
             unsigned spins = 0;

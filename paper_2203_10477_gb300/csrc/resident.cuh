@@ -681,7 +681,11 @@ struct Exchange {
                     }
             ok = __all_sync(kFull, ok);
         }
-        if (!ok) return false;
+        if (!ok) {
+            // (what this warp sent to a neighbour in the cluster lands while both are there)
+            if (cluster) __nanosleep(20000);
+            return false;
+        }
         __syncwarp();
         {
             const Real *su = hu + par * hstep, *sw = hw + par * hstep;

@@ -519,7 +519,8 @@ __global__ void __launch_bounds__(32 * radj_max_warps<Real>(P), 1)
                 ex.hstep = s_lane[64];
                 ex.hu = area0 + s_lane[96];
                 ex.hw = area0 + s_lane[128];
-                ok = ex.swap(prm.x, l, lw, done / prm.E - 1, false);
+                const int x_no = done / prm.E - 1;
+                ok = ex.swap(prm.x, l, lw, x_no, g == prm.inject_warp && x_no >= prm.inject_exchange);
                 if (!ok) {
                     latch_error(prm.x.err, kDevTimeoutFlag, g, k, 1);
                     break;
@@ -528,6 +529,8 @@ __global__ void __launch_bounds__(32 * radj_max_warps<Real>(P), 1)
             n0 = n0_next;
             len = len_next;
         }
+        // (a sweep that was given up has a part's copies on the way)
+        asm volatile("cp.async.wait_all;" ::: "memory");
         double sum = acc;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(kFull, sum, o);

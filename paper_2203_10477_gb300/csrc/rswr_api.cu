@@ -100,6 +100,8 @@ struct Engine {
     int64_t ck_spacing = 0;  // adjoint checkpoint spacing in spans (0: automatic)
     int S = 1, H = 4, W = 0, core = 0, P = 0, NT = 0;
     int inject_tile = -1, inject_span = -1;
+    // the test hook on an exchange of a sweep or a grid barrier (RSWR_INJECT_SWEEP)
+    bool inject_sweep() const { return inject_tile >= 0 && inject_span >= RSWR_INJECT_SWEEP; }
     int pass = 1;           // steps of a launch's span: whole spans of S (layout)
     bool span_set = false;  // the caller chose S
     bool is_plan = true;
@@ -1619,7 +1621,7 @@ bool radj_choose(Engine* e, int64_t T, RadjPlan* best)
                     c.cluster = cl == 1;
                     c.per_cta = per;
                     c.grid = (c.nw + per - 1) / per;
-                    if (cl && c.grid > 16) continue;
+                    if (cl && (c.grid > 16 || e->inject_sweep())) continue;
                     // model (ns per level, fitted as res_cost): eight FP64 operations of 64 clocks
                     // per point and warp; FP32 12 P + 45 issue slots, a chain of two steps
                     const double clk = 1.0 / 1.92;
@@ -1806,6 +1808,8 @@ rswr_status adjoint_resident(Engine* e, int64_t T, const int64_t* j_r, const voi
     prm.split = rj.split;
     prm.parts = (int32_t)parts;
     prm.E = rj.E;
+    prm.inject_warp = e->inject_sweep() ? e->inject_tile : -1;
+    prm.inject_exchange = e->inject_span - RSWR_INJECT_SWEEP;
     RSWR_CUDA(radj_launch(rj.v, &prm, rj.grid, 32 * rj.per_cta, smem, rj.cluster, s));
     if (grad_a) {
         const int64_t* d_red = reinterpret_cast<const int64_t*>(d_tab + b_prob + b_warp);
@@ -2493,7 +2497,7 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
     PaperRunChoice rc;
     std::vector<PaperPiece> pieces;
     int64_t npair = 0;
-    if (sizeof(Real) == 4 && T > 0 && e->inject_tile < 0 &&
+    if (sizeof(Real) == 4 && T > 0 && (e->inject_tile < 0 || e->inject_sweep()) &&
         paper_run_choose(e->form, nx, ov, cap, tau_max, e->num_sms, &rc))
         pieces = paper_pieces(ph, cap, rc, &npair);
     // workspace: the zones' scratch pair, flux waveforms, tiles, span word
@@ -2622,6 +2626,8 @@ rswr_status run_paper(Engine* e, const Real* fA, const Real* fB, int64_t T, cons
             q.cap = (int32_t)cap;
             q.steps = (int32_t)std::min<int64_t>(tau, T);
             q.warp_values = rc.warp_values;
+            q.inject_cta = e->inject_sweep() ? e->inject_tile : -1;
+            q.inject_barrier = e->inject_span - RSWR_INJECT_SWEEP;
             pp.u = static_cast<Real*>(e->q0[0]) + ph.base;
             pp.w = static_cast<Real*>(e->q1[0]) + ph.base;
             // (the last span's pieces are stored while others of it still read the samples)

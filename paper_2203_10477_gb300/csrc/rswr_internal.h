@@ -208,6 +208,7 @@ struct PaperRun {
     int64_t spans_cap, npiece, npair;  // pieces: npair pairs, then single ones
     int64_t T, beta_m, swap_u, swap_w;  // swap: from the first to the second state buffer
     int32_t cap, steps, warp_values;
+    int32_t inject_cta, inject_barrier;  // test hook (-1: off)
 };
 
 struct PaperRunChoice {
@@ -311,6 +312,7 @@ struct ResAdjParams {
     int32_t split;      // > 0: a span in two parts, the first of so many steps
     int32_t parts;      // parts of the sweep (state x at the start of part x)
     int32_t E;          // spans between two exchanges (halo >= E span)
+    int32_t inject_warp, inject_exchange;  // test hook (-1: off)
 };
 
 struct VariantInfo {

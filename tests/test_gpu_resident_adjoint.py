@@ -48,6 +48,8 @@ def test_sums_over_spans_leave_fp32s_range(R, oracle_mod, nx):
     assert torch.equal(got[0]["grad_fA"], got[1]["grad_fA"])
 
 
+SWEEP = 0x40000000  # RSWR_INJECT_SWEEP
+
 
 def gradient(R, dtype, nx, T=300, jr=200):
     td = torch.float64 if dtype == F64 else torch.float32
@@ -78,3 +80,43 @@ def test_gradients_run_without_the_hook(R, dtype):
         again = keep()
         plan.check()
         assert torch.equal(again["u"], kept["u"]) and torch.equal(again["recv"], kept["recv"])
+
+
+@pytest.mark.parametrize("dtype,nx", [(F32, 20001), (F32, 1 << 20), (F64, 20001), (F64, 60001)])
+@pytest.mark.parametrize("exchange", [0, 2])
+def test_an_adjoint_exchange_that_never_comes(R, dtype, nx, exchange):
+    """The neighbours' waits run out, every warp leaves the sweep, the status says so,
+    and the next gradient is exact."""
+    plan, grad, keep = gradient(R, dtype, nx)
+    ref = grad()
+    plan.set_wait_limit(0.2)
+    plan.inject_missing_flag(1, SWEEP + exchange)
+    for kept in (False, True):
+        if kept:
+            keep()
+            plan.check()  # (the forward run is not affected)
+        grad()
+        with pytest.raises(R.RSWRError) as ei:
+            plan.check()
+        assert ei.value.status == 6
+    plan.inject_missing_flag(-1, 0)
+    got = grad()
+    plan.check()
+    assert same(got, ref)
+
+
+@pytest.mark.parametrize("barrier", [0, 1, 4])
+def test_a_grid_barrier_of_the_paper_run_that_never_opens(R, barrier):
+    nx, T = 60001, 150
+    fA = torch.as_tensor(inputs.rng(3).standard_normal(T + 1).astype(np.float32), device="cuda")
+    plan = R.Plan(0.0, 1.0, 1.0, nx, 0.9 / (nx - 1), 30, 64, dtype=F32)
+    ref = plan.run_paper(fA, None, T)
+    assert len(ref["spans"]) > 3
+    plan.set_wait_limit(0.2)
+    plan.inject_missing_flag(1, SWEEP + barrier)
+    with pytest.raises(R.RSWRError) as ei:
+        plan.run_paper(fA, None, T)
+    assert ei.value.status == 6
+    plan.inject_missing_flag(-1, 0)
+    got = plan.run_paper(fA, None, T)
+    assert torch.equal(got["u"], ref["u"]) and list(got["spans"]) == list(ref["spans"])
