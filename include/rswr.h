@@ -152,9 +152,9 @@ typedef struct rswr_plan_info {
 rswr_status rswr_plan_get_info(rswr_plan_t plan, rswr_plan_info* info);
 
 /* Steps per span, 1 <= S <= floor(overlap/2) (else EOVERLAP).  A span that was
- * set is also what one launch or ticket advances; an FP32 plan as created
- * (S = floor(overlap/2)) or tuned runs as many whole spans per pass as 32 steps
- * hold.  The results are the same. */
+ * set, or that the autotuner chose below floor(overlap/2), is also what one launch
+ * or ticket advances; an FP32 plan with S = floor(overlap/2) as created runs as many
+ * whole spans per pass as 32 steps hold.  The results are the same. */
 rswr_status rswr_plan_set_span(rswr_plan_t plan, int32_t S);
 
 /* Kernel variant (points per thread x threads per CTA) for the plan's dtype

@@ -103,7 +103,7 @@ struct Engine {
     // the test hook on an exchange of a sweep or a grid barrier (RSWR_INJECT_SWEEP)
     bool inject_sweep() const { return inject_tile >= 0 && inject_span >= RSWR_INJECT_SWEEP; }
     int pass = 1;           // steps of a launch's span: whole spans of S (layout)
-    bool span_set = false;  // the caller chose S
+    bool span_set = false;  // the caller chose S, or the autotuner a shorter one
     bool is_plan = true;
     bool part = false;  // a part [lo, hi) of a larger grid (rswr_plan_create_part)
 
@@ -2287,28 +2287,31 @@ void tune_save()
     std::fclose(f);
 }
 
+int span_limit(const Engine* e)
+{
+    int S = 1 << 30;
+    for (const ProbHost& p : e->probs) S = std::min(S, p.ov / 2);
+    return std::min(S, kSpanCap);
+}
+
 rswr_status apply_choice(Engine* e, const TuneChoice& c)
 {
     const int oldS = e->S, oldV = e->variant;
+    const bool old_set = e->span_set;
     e->S = c.S;
     e->variant = c.variant;
+    e->span_set = c.S < span_limit(e);  // (timed as it is: one span to a pass)
     rswr_status st = layout(e);
     if (st != RSWR_OK) {
         e->S = oldS;
         e->variant = oldV;
+        e->span_set = old_set;
         layout(e);
         return st;
     }
     e->mode = c.mode;
     e->chosen = true;
     return RSWR_OK;
-}
-
-int span_limit(const Engine* e)
-{
-    int S = 1 << 30;
-    for (const ProbHost& p : e->probs) S = std::min(S, p.ov / 2);
-    return std::min(S, kSpanCap);
 }
 
 rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cudaStream_t s, bool use_cache)
@@ -2367,7 +2370,6 @@ rswr_status autotune_engine(Engine* e, int64_t probe_steps, int32_t* variant, cu
             if (vi.resident && !res_choose(e, vi.P, S, kResMaxHalo, false, false, false, &fit)) continue;
             for (int mode = 0; mode < (vi.resident ? 1 : 2); ++mode) {  // (one mode for resident windows)
                 if (apply_choice(e, TuneChoice{v, mode, S}) != RSWR_OK) continue;
-                if (S < S_max && e->pass >= S_max) continue;  // (the same passes as with S_max)
                 if (run_engine(e, r, s) != RSWR_OK) continue;  // warm-up (and graph capture)
                 RSWR_CUDA(cudaEventRecord(a, s));
                 rswr_status st = run_engine(e, r, s);
