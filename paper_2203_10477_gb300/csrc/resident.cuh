@@ -98,6 +98,19 @@ __device__ __forceinline__ void st_shared_if16(bool on, const float* d, const fl
                  : "memory");
 }
 
+__device__ __forceinline__ void st_global_if(bool on, float* d, float a)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.f32 [%1], %2;\n\t}" ::"r"((uint32_t)on), "l"(d),
+                 "f"(a)
+                 : "memory");
+}
+__device__ __forceinline__ void st_global_if(bool on, double* d, double a)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.f64 [%1], %2;\n\t}" ::"r"((uint32_t)on), "l"(d),
+                 "d"(a)
+                 : "memory");
+}
+
 // Warps of a CTA at most: 16 (one CTA then holds an SM's whole register file),
 // 8 where a lane's points fill more than 64 registers.
 template <typename Real>
@@ -116,6 +129,24 @@ __host__ __device__ inline size_t warp_values(int H, int P, int probe_rows)
     const int row = kRing * kRowLanes<Real>(P) * P;
     n += (size_t)probe_rows * (row > 2 * kFastRing ? row : 2 * kFastRing);
     return (n + 3) / 4 * 4;
+}
+
+// A probe on one of a lane's own points, where a warp has more than two.
+template <typename Real>
+struct LaneProbe {
+    Real* out;
+    int64_t stride;
+    Real scale;
+    int32_t nmax;
+    int32_t code;  // 2 (register + 1) + kind; a node beside the window: register -1 or P; -1: none
+};
+
+// Records of every lane that the row buffers of two probes hold.
+template <typename Real>
+__host__ __device__ constexpr int max_rounds(int P)
+{
+    const int row = kRing * kRowLanes<Real>(P) * P;
+    return 2 * (row > 2 * kFastRing ? row : 2 * kFastRing) * (int)sizeof(Real) / (32 * (int)sizeof(LaneProbe<Real>));
 }
 
 // The samples of a warp's one special point (a node's value, a source's
@@ -709,7 +740,9 @@ struct Exchange {
     }
 };
 
-template <typename Real, int FORM, int P>
+// DENSE: compiled with the records of windows that hold many probes (runs without
+// such a window pay 2 % for the code: 2^20 points, 406 -> 413 us).
+template <typename Real, int FORM, int P, bool DENSE>
 __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(const __grid_constant__ ResParams<Real> prm)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -818,6 +851,12 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
     // or last register (the host shifts a window for that): the owner drops the
     // value (flux: both neighbours) into a small buffer every level.  Else the
     // first two through rows of all the registers, further ones directly.
+    // DENSE: of more than two every lane holds the records of those on its own
+    // points and stores their values each level, all lanes at once: a level costs
+    // four instructions per register however many there are.  (One by one from the
+    // table, 0.36 us each on a window of 1024 points, they lost to tickets from three
+    // on: 2^20 points in 1497 subdomains, all traces, 512 steps 795 us, with tickets
+    // 723, this way 488.)  Only where a lane has more than fit are they taken so.
     constexpr int RL = kRowLanes<Real>(P);
     const int np = wd.probe_end - wd.probe_begin;
     const ProbeDev<Real>* const probes = prm.probes + wd.probe_begin;
@@ -842,6 +881,59 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
             pr[q] = pos - pl[q] * P;
         }
     if (fast) pl[0] = pl[1] = -64;
+    int rounds = 0;  // records of a lane
+    LaneProbe<Real>* const recs = reinterpret_cast<LaneProbe<Real>*>(ring) + lane;  // [round][32]
+    if (DENSE && slow) {
+        // (the probes are sorted by point)
+        auto below = [&](int64_t j) {
+            int a = 0, b = np;
+            while (a < b) {
+                const int m = (a + b) >> 1;
+                if (probes[m].gidx < j) a = m + 1;
+                else b = m;
+            }
+            return a;
+        };
+        const int from = below(j0 - (spec == kNodeLeft && lane == 0 ? 1 : 0));
+        const int n = below(j0 + P + (spec == kNodeRight && lane == 31 ? 1 : 0)) - from;
+        rounds = __reduce_max_sync(kFull, n);
+        if (rounds <= max_rounds<Real>(P)) {
+            for (int t = 0; t < rounds; ++t) {
+                LaneProbe<Real> q{};
+                q.code = -1;
+                if (t < n) {
+                    const ProbeDev<Real> p = probes[from + t];
+                    q.out = p.out;
+                    q.stride = p.stride;
+                    q.scale = p.scale;
+                    q.nmax = (int32_t)(p.nmax < 0x7fffffff ? p.nmax : 0x7fffffff);
+                    q.code = 2 * ((int)p.gidx - j0 + 1) + (p.kind != 0 ? 1 : 0);
+                }
+                recs[32 * t] = q;
+            }
+            slow = false;
+            pl[0] = pl[1] = -64;
+        } else {
+            rounds = 0;
+        }
+    }
+    // level n of the points that have records
+    auto put_records = [&](const Real(&x)[P], Real lft, Real rgt, int n) {
+        for (int t = 0; t < rounds; ++t) {
+            const LaneProbe<Real> q = recs[32 * t];
+            const int r = (q.code >> 1) - 1;
+            Real um = lft, uc = r < 0 ? lft : rgt, up = rgt;
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+                if (i == r) {
+                    uc = x[i];
+                    um = i > 0 ? x[i > 0 ? i - 1 : 0] : lft;
+                    up = i < P - 1 ? x[i < P - 1 ? i + 1 : 0] : rgt;
+                }
+            const Real val = q.code & 1 ? rsub(up, um) : uc;
+            st_global_if(q.code >= 0 && n <= q.nmax, q.out + n * q.stride, rmul(val, q.scale));
+        }
+    };
     // level n into the fast probes' buffers [probe][level mod kFastRing]{value or right, left}
     auto put_fast = [&](const Real(&x)[P], Real lft, Real rgt, int n) {
 #pragma unroll
@@ -1004,7 +1096,10 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
             } else if (fast) {
                 advance([&](const Real(&x)[P], Real l, Real r, int s) { put_fast(x, l, r, (int)b0 + s); });
             } else {
-                advance([&](const Real(&x)[P], Real, Real, int s) { put_rows(x, (int)b0 + s); });
+                advance([&](const Real(&x)[P], Real l, Real r, int s) {
+                    if (DENSE && rounds) put_records(x, l, r, (int)b0 + s);
+                    else put_rows(x, (int)b0 + s);
+                });
             }
             if (np && ((int)(b0 + n) & (probe_levels - 1)) == 0) flush(b0 + n);
             if (prm.ck0 && (part_left -= n) == 0) {
@@ -1028,11 +1123,12 @@ __global__ void __launch_bounds__(32 * max_warps<Real>(P), 1) resident_kernel(co
 
     // ---- level T: probes and the state pair
     if (np > 0) {
-        if (fast) {
+        if (fast || (DENSE && rounds)) {
             Real l = __shfl_up_sync(kFull, u[P - 1], 1), r = __shfl_down_sync(kFull, u[0], 1);
             if (spec == kNodeLeft && lane == 0) l = node_sample(pb.fA, prm.T);
             if (spec == kNodeRight && lane == 31) r = node_sample(pb.fB, prm.T);
-            put_fast(u, l, r, (int)prm.T);
+            if (fast) put_fast(u, l, r, (int)prm.T);
+            else put_records(u, l, r, (int)prm.T);
         } else {
             put_rows(u, (int)prm.T);
         }

@@ -11,14 +11,16 @@ using namespace resident;
 
 struct Entry {
     int dtype, form, P;
-    const void* fn;
+    const void* fn;        // at most two probes to a window, or few points with more
+    const void* fn_dense;
 };
 
 template <typename Real, int FORM, int P>
 Entry entry()
 {
     return Entry{sizeof(Real) == 8 ? kF64 : kF32, FORM, P,
-                 reinterpret_cast<const void*>(&resident_kernel<Real, FORM, P>)};
+                 reinterpret_cast<const void*>(&resident_kernel<Real, FORM, P, false>),
+                 res_dense_kernel(sizeof(Real) == 8 ? kF64 : kF32, P)};
 }
 
 const Entry* find(int dtype, int form, int P)
@@ -51,20 +53,21 @@ size_t res_slot_bytes(int dtype, int H)
     return sizeof(ulonglong2) * 4 * (size_t)H * (dtype == kF64 ? slot_words<double> : slot_words<float>);
 }
 
-cudaError_t res_occupancy(int dtype, int form, int P, int threads, size_t smem, int* ctas_per_sm)
+cudaError_t res_occupancy(int dtype, int form, int P, bool dense, int threads, size_t smem, int* ctas_per_sm)
 {
     *ctas_per_sm = 0;
     const Entry* e = find(dtype, form, P);
     if (!e) return cudaSuccess;
+    const void* const fn = dense ? e->fn_dense : e->fn;
     int dev = 0, per_block = 0;
     cudaError_t st = cudaGetDevice(&dev);
     if (st == cudaSuccess) st = cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (st != cudaSuccess) return st;
     per_block -= 2048;  // (room for the static part)
     if (smem > (size_t)per_block) return cudaSuccess;
-    st = cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, per_block);
+    st = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, per_block);
     if (st != cudaSuccess) return st;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, e->fn, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, threads, smem);
 }
 
 namespace {
@@ -115,18 +118,18 @@ cudaError_t res_launch_kernel(const void* fn, const void* params, int grid, int 
     return cudaLaunchKernelExC(&c, fn, args);
 }
 
-cudaError_t res_clusters(int dtype, int form, int P, int grid, int threads, size_t smem, int* clusters)
+cudaError_t res_clusters(int dtype, int form, int P, bool dense, int grid, int threads, size_t smem, int* clusters)
 {
     *clusters = 0;
     const Entry* e = find(dtype, form, P);
-    return e ? res_kernel_clusters(e->fn, grid, threads, smem, clusters) : cudaSuccess;
+    return e ? res_kernel_clusters(dense ? e->fn_dense : e->fn, grid, threads, smem, clusters) : cudaSuccess;
 }
 
-cudaError_t res_launch(int dtype, int form, int P, const void* params, int grid, int threads, size_t smem,
+cudaError_t res_launch(int dtype, int form, int P, bool dense, const void* params, int grid, int threads, size_t smem,
                        bool cluster, cudaStream_t s)
 {
     const Entry* e = find(dtype, form, P);
-    return e ? res_launch_kernel(e->fn, params, grid, threads, smem, cluster, s) : cudaErrorInvalidValue;
+    return e ? res_launch_kernel(dense ? e->fn_dense : e->fn, params, grid, threads, smem, cluster, s) : cudaErrorInvalidValue;
 }
 
 }  // namespace rswr

@@ -932,7 +932,7 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool slack, b
             r.grid = (r.nw + r.per_cta - 1) / r.per_cta;
             int values = 0, occ = 0;
             const size_t smem = res_smem_bytes(e->dtype, P, H, r.per_cta, probes ? 2 : 0, &values);
-            if (res_occupancy(e->dtype, e->form, P, 32 * r.per_cta, smem, &occ) != cudaSuccess) {
+            if (res_occupancy(e->dtype, e->form, P, false, 32 * r.per_cta, smem, &occ) != cudaSuccess) {
                 cudaGetLastError();
                 continue;
             }
@@ -950,8 +950,8 @@ bool res_search(const Engine* e, int want_P, int S, int max_spans, bool slack, b
                 if (grid > 16) continue;
                 const size_t sm = res_smem_bytes(e->dtype, P, H, per_cta, probes ? 2 : 0, &values);
                 int fit = 0;
-                if (res_occupancy(e->dtype, e->form, P, 32 * per_cta, sm, &occ) != cudaSuccess || occ < 1 ||
-                    res_clusters(e->dtype, e->form, P, grid, 32 * per_cta, sm, &fit) != cudaSuccess || fit < 1) {
+                if (res_occupancy(e->dtype, e->form, P, false, 32 * per_cta, sm, &occ) != cudaSuccess || occ < 1 ||
+                    res_clusters(e->dtype, e->form, P, false, grid, 32 * per_cta, sm, &fit) != cudaSuccess || fit < 1) {
                     cudaGetLastError();
                     continue;
                 }
@@ -1329,10 +1329,24 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     prm.inject_chunk = (int32_t)((int64_t)e->inject_span * e->S / rp.S);
     int values = 0;
     const size_t smem = res_smem_bytes(e->dtype, rp.P, rp.H, rp.per_cta, r.probes.empty() ? 0 : 2, &values);
+    // more than two probes in some window: the kernel with their records, where the
+    // cut fits it as well
+    bool dense = false;
+    for (const ResWarp& w : warps) dense = dense || w.probe_end - w.probe_begin > 2;
+    if (dense) {
+        int fit = 0;
+        if (res_occupancy(e->dtype, e->form, rp.P, true, 32 * rp.per_cta, smem, &fit) != cudaSuccess ||
+            (int64_t)fit * e->num_sms < rp.grid ||
+            (rp.cluster && (res_clusters(e->dtype, e->form, rp.P, true, rp.grid, 32 * rp.per_cta, smem, &fit) != cudaSuccess ||
+                            fit < 1))) {
+            cudaGetLastError();
+            dense = false;
+        }
+    }
     prm.x = res_exchange(e, rp.H, values, rp.cluster);
     // (the events time runs, not a gradient's own forward sweep)
     if (!keep && (st = record_event(e->ev_start, s)) != RSWR_OK) return st;
-    RSWR_CUDA(res_launch(e->dtype, e->form, rp.P, &prm, rp.grid, 32 * rp.per_cta, smem, rp.cluster, s));
+    RSWR_CUDA(res_launch(e->dtype, e->form, rp.P, dense, &prm, rp.grid, 32 * rp.per_cta, smem, rp.cluster, s));
     if (!keep && (st = record_event(e->ev_stop, s)) != RSWR_OK) return st;
     const size_t state = sizeof(Real) * (size_t)e->packed_len;
     if (aside && r.out0) RSWR_CUDA(cudaMemcpyAsync(r.out0, e->d_scratch[0], state, cudaMemcpyDeviceToDevice, s));

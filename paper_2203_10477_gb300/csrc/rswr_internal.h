@@ -339,11 +339,13 @@ cudaError_t span_launch(int v, const void* params, int grid, cudaStream_t s);
 size_t res_smem_bytes(int dtype, int P, int H, int warps_per_cta, int probe_rows, int* warp_values);
 int res_max_warps(int dtype, int P);      // warps of a CTA at most
 size_t res_slot_bytes(int dtype, int H);  // exchange slots of one CTA
-cudaError_t res_occupancy(int dtype, int form, int P, int threads, size_t smem, int* ctas_per_sm);
+// dense: the kernel for runs with more than two probes in some window
+cudaError_t res_occupancy(int dtype, int form, int P, bool dense, int threads, size_t smem, int* ctas_per_sm);
 // clusters of `grid` CTAs that fit on the GPU at once
-cudaError_t res_clusters(int dtype, int form, int P, int grid, int threads, size_t smem, int* clusters);
-cudaError_t res_launch(int dtype, int form, int P, const void* params, int grid, int threads, size_t smem,
+cudaError_t res_clusters(int dtype, int form, int P, bool dense, int grid, int threads, size_t smem, int* clusters);
+cudaError_t res_launch(int dtype, int form, int P, bool dense, const void* params, int grid, int threads, size_t smem,
                        bool cluster, cudaStream_t s);
+const void* res_dense_kernel(int dtype, int P);  // resident_dense_kernel.cu
 
 // any kernel over resident warps: one cooperative grid, or one cluster
 cudaError_t res_kernel_clusters(const void* fn, int grid, int threads, size_t smem, int* clusters);
