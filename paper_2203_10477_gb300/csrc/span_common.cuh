@@ -370,24 +370,8 @@ __device__ __forceinline__ void record_probes(const Real (&u)[P], Real lft, Real
     }
 }
 
-// A tile's probes staged in shared memory once per tile; each thread keeps the
-// indices of (at most two) probes whose point it owns.
+// A tile's probes staged in shared memory once per tile.
 constexpr int kTileProbes = 16;
-
-template <typename Real, int P>
-__device__ __forceinline__ void owned_probes(const ProbeDev<Real>* sp, int np, int64_t wabs, int tb, int rlo, int rhi,
-                                             int& q0, int& q1)
-{
-    q0 = -1;
-    q1 = -1;
-    for (int q = 0; q < np; ++q) {
-        const int64_t li = sp[q].gidx - wabs - (int64_t)tb;
-        if (li >= rlo && li < rhi) {
-            if (q0 < 0) q0 = q;
-            else q1 = q;
-        }
-    }
-}
 
 // u[r-1], u[r], u[r+1] of a register index r known only at run time: a
 // binary tree of branches on r (log2 P compares, then three moves) instead of
