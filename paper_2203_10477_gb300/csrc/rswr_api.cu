@@ -85,6 +85,7 @@ struct ResPlan {
     bool slack = false;        // windows leave room to put a source or probe on an end register
     bool linked = false;       // some problem has more than one warp
     bool cluster = false;      // the grid is one thread-block cluster
+    bool dense = false;        // the kernel for many probes in a window fits as well
     double cost = 0.0;         // model: ns per step
 };
 
@@ -980,6 +981,16 @@ bool res_choose(Engine* e, int want_P, int S, int max_spans, bool sources, bool 
         if (!res_search(e, want_P, S, max_spans, slack, probes, kept, &r) &&
             !(slack && res_search(e, want_P, S, max_spans, false, probes, kept, &r)))
             r.nw = 0;
+        if (probes && r.nw > 0) {
+            int values = 0, fit = 0;
+            const size_t smem = res_smem_bytes(e->dtype, r.P, r.H, r.per_cta, 2, &values);
+            r.dense = res_occupancy(e->dtype, e->form, r.P, true, 32 * r.per_cta, smem, &fit) == cudaSuccess &&
+                      (int64_t)fit * e->num_sms >= r.grid;
+            if (r.dense && r.cluster)
+                r.dense = res_clusters(e->dtype, e->form, r.P, true, r.grid, 32 * r.per_cta, smem, &fit) == cudaSuccess &&
+                          fit >= 1;
+            if (!r.dense) cudaGetLastError();
+        }
         it = e->res_plans.emplace(key, r).first;
     }
     *best = it->second;
@@ -1017,6 +1028,18 @@ Range probe_range(const ProbeReq& q, size_t es)
     return Range(static_cast<char*>(q.out) + std::min<int64_t>(last, 0), (size_t)std::llabs(last) + es);
 }
 
+// The smallest range that holds all of a run's records.
+Range probes_range(const RunReq& r, size_t es)
+{
+    Range all(nullptr, 0);
+    for (const ProbeReq& q : r.probes) {
+        const Range o = probe_range(q, es);
+        all.lo = all.hi == 0 ? o.lo : std::min(all.lo, o.lo);
+        all.hi = std::max(all.hi, o.hi);
+    }
+    return all;
+}
+
 // Whether the final state may not go straight to out0 / out1 while the run's
 // kernel still works: some of what it reads lies there (a run in place, say), or
 // another output of it, which the state replaces.
@@ -1031,9 +1054,11 @@ bool outputs_meet(const Engine* e, const RunReq& r)
                            Range(r.fB, samples), Range(e->usrc_samples, es * (size_t)(rows * e->usrc_pitch))};
     const Range out[] = {Range(r.out0, state), Range(r.out1, state)};
     if (out[0].meets(out[1])) return true;
+    const Range records = probes_range(r, es);
     for (const Range& o : out) {
         for (const Range& x : reads)
             if (o.meets(x)) return true;
+        if (!o.meets(records)) continue;
         for (const ProbeReq& q : r.probes)
             if (o.meets(probe_range(q, es))) return true;
     }
@@ -1045,9 +1070,12 @@ bool outputs_meet(const Engine* e, const RunReq& r)
 bool probes_meet_state(const Engine* e, const RunReq& r)
 {
     const size_t es = e->esize(), state = es * (size_t)e->packed_len;
-    if (r.q0)
-        for (const ProbeReq& q : r.probes)
-            if (probe_range(q, es).meets(Range(r.q0, state)) || probe_range(q, es).meets(Range(r.q1, state))) return true;
+    const Range in0(r.q0, state), in1(r.q0 ? r.q1 : nullptr, state);
+    if (!r.q0 || r.probes.empty()) return false;
+    const Range records = probes_range(r, es);
+    if (!records.meets(in0) && !records.meets(in1)) return false;
+    for (const ProbeReq& q : r.probes)
+        if (probe_range(q, es).meets(in0) || probe_range(q, es).meets(in1)) return true;
     return false;
 }
 
@@ -1329,20 +1357,10 @@ rswr_status res_run(Engine* e, const RunReq& r, const ResPlan& rp, const ResKeep
     prm.inject_chunk = (int32_t)((int64_t)e->inject_span * e->S / rp.S);
     int values = 0;
     const size_t smem = res_smem_bytes(e->dtype, rp.P, rp.H, rp.per_cta, r.probes.empty() ? 0 : 2, &values);
-    // more than two probes in some window: the kernel with their records, where the
-    // cut fits it as well
+    // more than two probes in some window: the kernel with their records
     bool dense = false;
-    for (const ResWarp& w : warps) dense = dense || w.probe_end - w.probe_begin > 2;
-    if (dense) {
-        int fit = 0;
-        if (res_occupancy(e->dtype, e->form, rp.P, true, 32 * rp.per_cta, smem, &fit) != cudaSuccess ||
-            (int64_t)fit * e->num_sms < rp.grid ||
-            (rp.cluster && (res_clusters(e->dtype, e->form, rp.P, true, rp.grid, 32 * rp.per_cta, smem, &fit) != cudaSuccess ||
-                            fit < 1))) {
-            cudaGetLastError();
-            dense = false;
-        }
-    }
+    if (rp.dense)
+        for (const ResWarp& w : warps) dense = dense || w.probe_end - w.probe_begin > 2;
     prm.x = res_exchange(e, rp.H, values, rp.cluster);
     // (the events time runs, not a gradient's own forward sweep)
     if (!keep && (st = record_event(e->ev_start, s)) != RSWR_OK) return st;
