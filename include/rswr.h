@@ -241,6 +241,8 @@ rswr_status rswr_plan_check(rswr_plan_t plan, void* stream, int32_t* code, int32
  *            flux = (u_{j+1} - u_{j-1}) * inv2dx.
  *   j_r, recv  receiver: recv[n] = u^n_{j_r}, n = 0..T (recv may be NULL; j_r
  *            ignored then).
+ * out0 and out1 may lie where the run reads (a run in place, or with the pair
+ * swapped): they are written when everything has been read, out1 after out0.
  * Errors: EINVAL, ECUDA.  Device-side timeouts: see rswr_plan_check.
  */
 rswr_status rswr_run(rswr_plan_t plan, const void* fA, const void* fB, int64_t T, const void* q0, const void* q1,
@@ -316,7 +318,8 @@ rswr_status rswr_run_keep(rswr_plan_t plan, const void* fA, const void* fB, int6
  * state is kept when they fit in half of the free device memory (one forward
  * sweep, then one adjoint launch over all spans -- both on resident warps when
  * the grid fits on the chip and the plan is as created or on a resident
- * variant, else persistent), else
+ * variant, else persistent; resident FP32 sweeps of more than about half a
+ * million points keep a state every 8 levels, twice as many), else
  * one checkpoint every ceil(sqrt(#spans)) spans with the states of each
  * segment recomputed before its spans are processed
  * (rswr_plan_set_checkpoint_spacing overrides).
@@ -466,10 +469,14 @@ rswr_status rswr_variant_get_tiling(int32_t v, int32_t* warp_halo, int32_t* wind
  *                                 moves the windows (tickets, TMA, flags);
  *   RSWR_VARIANT_RESIDENT         every warp keeps its window on chip for the
  *                                 whole run and only halo strips are exchanged,
- *                                 every so many spans; a grid that is a little
- *                                 too large runs on the default variant, one of
- *                                 more than 13312 FP32 (3968 FP64) points per SM
- *                                 is refused by rswr_run with RSWR_ENOTSUP.  A plan or batch as it was
+ *                                 every so many spans; runs that this does not
+ *                                 cover (a grid that is a little too large, a
+ *                                 record over the initial state, spans beyond 64
+ *                                 steps) take the default variant's tiles, which
+ *                                 rswr_plan_get_info reports; a grid of more than
+ *                                 13312 FP32 (3968 FP64) points per SM that does
+ *                                 not fit is refused by rswr_run with
+ *                                 RSWR_ENOTSUP.  A plan or batch as it was
  *                                 created runs this way by itself when it fits
  *                                 (same results); one whose variant, span or
  *                                 mode was set, or chosen by the autotuner,

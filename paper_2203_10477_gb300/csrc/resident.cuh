@@ -28,9 +28,9 @@
 //   * a probe's window is placed so that its point is a lane's first or last
 //     register; the lane drops the value into a shared buffer every step, and the
 //     warp turns 32 levels into one coalesced store (elsewhere: rows of all the
-//     lane's registers).
-// The final state goes straight to the caller's arrays, the initial state
-// comes straight from them.
+//     lane's registers; more than two probes: a record per lane).
+// The initial state comes straight from the caller's arrays and the final state
+// goes straight to them, unless it would land on what the run still reads.
 //
 // Measured, whole runs, against the ticketed kernels (the last: against one CTA
 // per resident tile): 1001 FP64 points, 2000 steps 4636 -> 694 us; 8001 FP32, 2000

@@ -18,8 +18,8 @@
 // per warp and scheduler); FP32 the issue slots on full grids (about 12 P + 45
 // instructions per warp and level) and the chain of two steps and the exchange
 // on small ones.  Measured: 2^20 FP32 points, 2048 levels, 1.43 ms for this sweep;
-// a training step with it 4389 (persistent adjoint_kernel) -> 2816 us; the
-// gradient of 65539 FP64 points, 2048 levels, 13113 -> 4523 us.
+// a training step with it 4389 .. 4509 (persistent adjoint_kernel) -> 2673 .. 3137 us;
+// the gradient of 65539 FP64 points, 2048 levels, 13113 -> 4537 us.
 
 #include "resident.cuh"
 #include "tmem.cuh"

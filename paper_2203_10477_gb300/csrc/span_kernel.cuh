@@ -8,7 +8,8 @@
 //       halo points on each side -- into shared memory with 1-D TMA bulk
 //       copies and advances it S leapfrog steps in registers.  Each window end
 //       that is not a physical boundary is an input boundary whose flux is
-//       guessed (mirror ghost, zero flux).
+//       guessed: a mirror ghost (zero flux), or in the loops of free warp windows
+//       whatever the end lane's own shuffle returns (any guess is cut off).
 //   select  (Sec. 2.4, Waveform Time Span Theorem): the guessed edges corrupt
 //       one more point per step (discrete domain of dependence), so after
 //       S <= H steps the core is exact; select is the index range of the
